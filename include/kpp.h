@@ -113,12 +113,14 @@ typedef struct {
     uint32_t timeout_us;      /* persistent form: bound of each grid-barrier wait;
                                  0 = 2,000,000 us */
     int32_t smem_cache;       /* persistent form: -1 = no shared-memory point cache,
-                                 0 = as many rows as fit, > 0 = at most this many
-                                 rows per CTA */
+                                 0 = every row if they all fit (else passes that skip
+                                 rows, or as many rows as fit where those do not
+                                 apply: K < 8, rows under 16 bytes, more than one CTA
+                                 per SM), > 0 = at most this many rows per CTA */
     int32_t alternate;        /* persistent form: 0/1 = walk rows backwards on odd
                                  passes (L2 reuse), -1 = always forwards */
-    int32_t l2_policy;        /* persistent form, streamed rows: 0 = evict-last,
-                                 -1 = no hint, 2 = evict-first */
+    int32_t l2_policy;        /* persistent form, streamed rows of plans that read every
+                                 row: 0 = evict-last, -1 = no hint, 2 = evict-first */
     int32_t min_rows_per_cta; /* persistent form: smallest row block; 0 = 2048 */
     int32_t exact_draws;      /* 1 = decide every "prefix > t" comparison of every draw
                                  in FP64 (t = u * T as the FP64 product of the draw's
@@ -143,7 +145,7 @@ typedef struct {
                                     (one warp's contiguous share of a block) */
     int64_t cached_rows_per_cta; /* persistent form: rows kept in shared memory */
     int64_t smem_bytes;          /* dynamic shared memory per CTA */
-    int64_t workspace_bytes;     /* same as kpp_workspace_size */
+    int64_t workspace_bytes;     /* the least workspace kpp_seed accepts */
 } kpp_plan;
 
 /* Human-readable name of a status code (static string, never NULL). */
@@ -153,9 +155,12 @@ KPP_API const char *kpp_status_string(kpp_status status);
 KPP_API int32_t kpp_version(void);
 
 /*
- * Bytes of device workspace kpp_seed needs for this problem on the current
- * device (0 if the arguments are invalid).  The size depends on N, d, dtype,
- * the options and the device's SM count, not on the data.
+ * Bytes of device workspace for kpp_seed and this problem on the current
+ * device (0 if the arguments are invalid).  The size depends on N, d, K,
+ * dtype, the options and the device's SM count, not on the data.  Where D^2
+ * does not fit shared memory it holds a 16-bit label per point, which lets a
+ * pass skip the rows it cannot change; a workspace of kpp_describe's
+ * workspace_bytes leaves them out: the same results, every row read.
  */
 KPP_API size_t kpp_workspace_size(int64_t N, int32_t d, int32_t K, kpp_dtype dtype,
                           const kpp_options *opts);

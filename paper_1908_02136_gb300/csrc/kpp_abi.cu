@@ -8,6 +8,7 @@
 
 #include "kpp.h"
 #include "kpp_internal.h"
+#include "kpp_pass.cuh"
 
 namespace kpp {
 namespace {
@@ -15,6 +16,7 @@ namespace {
 constexpr size_t kAlign = 256;
 constexpr int kMaxDim = 4096;
 constexpr int kDefaultCtasPerSm = 4;
+constexpr int kPruneMinK = 8; // fewer passes than this read every row
 
 size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -42,8 +44,11 @@ struct Plan {
     int nblocks;
     int nseg;   // segments (warps) per block
     int64_t sw; // rows per super-iteration
+    bool prune; // persistent form: passes skip the rows they cannot change
     // workspace layout (byte offsets after the control block)
     size_t off_bsum, off_seg, off_slots;
+    size_t min_bytes; // without the labels of `prune` (a workspace that holds no
+                      // more than these gets the seeding that reads every row)
     size_t ws_bytes;
 };
 
@@ -65,7 +70,7 @@ void layout(Plan *pl, bool persistent)
         pl->off_seg = off;
         off += round_up(sizeof(float2) * (size_t)pl->nblocks * pl->nseg, kAlign);
     }
-    pl->ws_bytes = off;
+    pl->min_bytes = pl->ws_bytes = off;
 }
 
 kpp_status plan_streamed(int64_t N, int32_t d, int dt, const kpp_options &o, int sms, Plan *pl)
@@ -88,6 +93,7 @@ kpp_status plan_streamed(int64_t N, int32_t d, int dt, const kpp_options &o, int
     int64_t chunk = (N + target - 1) / target;
     chunk = (chunk + a - 1) / a * a;
     pl->form = KPP_FORM_STREAMED;
+    pl->prune = false;
     pl->chunk = chunk;
     pl->nblocks = (int)((N + chunk - 1) / chunk);
     pl->grid = pl->nblocks;
@@ -126,8 +132,9 @@ kpp_status plan_small(int64_t N, int32_t d, int dt, Plan *pl)
     pl->grid = 1;
     pl->nseg = small_threads() / 32;
     pl->sw = 1;
+    pl->prune = false;
     pl->off_bsum = pl->off_seg = pl->off_slots = sizeof(Control);
-    pl->ws_bytes = sizeof(Control);
+    pl->min_bytes = pl->ws_bytes = sizeof(Control);
     return KPP_OK;
 }
 
@@ -197,8 +204,29 @@ kpp_status plan_persistent_at(int64_t N, int32_t K, const kpp_options &o, int sm
         if (supers < 0)
             supers = 0;
     }
-    pl->pfn = d2_in_smem ? pl->pk.fn_smem : pl->pk.fn_global;
     pl->psmem = (size_t)(supers * unit + (d2_in_smem ? d2_bytes : 0));
+    // Passes that skip rows, unless the caller asked for a point cache or the
+    // whole block fits one (its passes then read no row from L2 at all).
+    // Below kPruneMinK passes too few come after the first seeds, which can
+    // skip little (10^6 x 32, K = 256: 0.99 of the rows are read at pass 1,
+    // 0.78 at 25, 0.26 at 128).
+    pl->prune = false;
+    if (pl->pk.prune_smem && K >= kPruneMinK && per_sm == 1 && o.smem_cache <= 0 &&
+        supers < seg_supers) {
+        const PruneLayout in = prune_layout(d2_bytes, chunk, K, true, nseg);
+        d2_in_smem = d2_in_smem && in.bytes <= budget;
+        const int64_t bytes =
+            d2_in_smem ? in.bytes : prune_layout(0, chunk, K, false, nseg).bytes;
+        pl->prune = bytes <= budget;
+        if (pl->prune) {
+            supers = 0;
+            pl->psmem = (size_t)bytes;
+        }
+    }
+    if (pl->prune)
+        pl->pfn = d2_in_smem ? pl->pk.prune_smem : pl->pk.prune_global;
+    else
+        pl->pfn = d2_in_smem ? pl->pk.fn_smem : pl->pk.fn_global;
     // static + dynamic shared memory above 48 KB needs the opt-in attribute
     if (cudaFuncSetAttribute(pl->pfn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)pl->psmem) != cudaSuccess)
@@ -220,6 +248,8 @@ kpp_status plan_persistent_at(int64_t N, int32_t K, const kpp_options &o, int sm
     pl->pargs.l2_hint = o.l2_policy == 0 ? 1 : (o.l2_policy == 2 ? 2 : 0);
     pl->pargs.timeout_ns = 1000ull * (o.timeout_us ? o.timeout_us : 2000000u);
     layout(pl, true);
+    if (pl->prune && !d2_in_smem)
+        pl->ws_bytes += round_up(sizeof(uint16_t) * (size_t)N, kAlign); // the labels
     return KPP_OK;
 }
 
@@ -310,7 +340,7 @@ kpp_status run_persistent(const Plan &pl, const Problem &p, cudaStream_t stream)
 {
     // the control block and both slot buffers start at zero: a zeroed slot
     // never carries the tag a pass waits for
-    if (cudaMemsetAsync(p.ctl, 0, pl.ws_bytes, stream) != cudaSuccess)
+    if (cudaMemsetAsync(p.ctl, 0, pl.min_bytes, stream) != cudaSuccess)
         return KPP_ERR_CUDA;
     return persistent_launch(pl.pfn, pl.grid, pl.psmem, p, pl.pargs, stream) == cudaSuccess
                ? KPP_OK
@@ -378,6 +408,13 @@ kpp_status run_streamed(const Plan &pl, const Problem &p, cudaStream_t stream, i
 bool aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
 } // namespace
+
+bool plan_skips_rows(int64_t N, int32_t d, int32_t K, kpp_dtype dtype, const kpp_options *opts)
+{
+    Plan pl;
+    return make_plan(N, d, K, (int)dtype, opts, &pl) == KPP_OK && pl.prune;
+}
+
 } // namespace kpp
 
 using namespace kpp;
@@ -437,7 +474,7 @@ kpp_status kpp_describe(int64_t N, int32_t d, int32_t K, kpp_dtype dtype,
     plan->grid = pl.grid;
     plan->rows_per_cta = pl.chunk;
     plan->rows_per_segment = (pl.chunk + pl.nseg - 1) / pl.nseg;
-    plan->workspace_bytes = (int64_t)pl.ws_bytes;
+    plan->workspace_bytes = (int64_t)pl.min_bytes;
     if (pl.form == KPP_FORM_SMALL) {
         plan->threads = small_threads();
         plan->launches = 1;
@@ -448,7 +485,7 @@ kpp_status kpp_describe(int64_t N, int32_t d, int32_t K, kpp_dtype dtype,
         plan->threads = persistent_threads();
         plan->launches = 1;
         plan->lanes_per_row = pl.pk.lanes;
-        plan->d2_in_smem = pl.pfn == pl.pk.fn_smem ? 1 : 0;
+        plan->d2_in_smem = pl.pfn == pl.pk.fn_smem || pl.pfn == pl.pk.prune_smem ? 1 : 0;
         plan->cached_rows_per_cta = pl.pargs.cache_supers * pl.nseg * pl.sw;
         plan->smem_bytes = (int64_t)pl.psmem;
     } else {
@@ -477,8 +514,15 @@ kpp_status kpp_seed(const void *points, const float *row_scales, int64_t N, int3
     kpp_status st = make_plan(N, d, K, dt, opts, &pl);
     if (st != KPP_OK)
         return st;
-    if (!workspace || !aligned(workspace, kAlign) || workspace_bytes < pl.ws_bytes)
+    if (!workspace || !aligned(workspace, kAlign) || workspace_bytes < pl.min_bytes)
         return KPP_ERR_WORKSPACE;
+    if (pl.prune && workspace_bytes < pl.ws_bytes) {
+        // no room for the labels (only D^2 in the output array needs it): the
+        // kernel that reads every row, with the same blocks
+        pl.prune = false;
+        pl.pfn = pl.pk.fn_global;
+        pl.psmem = 0;
+    }
     Problem p;
     std::memset(&p, 0, sizeof(p));
     p.points = points;
@@ -502,6 +546,8 @@ kpp_status kpp_seed(const void *points, const float *row_scales, int64_t N, int3
     if (pl.form == KPP_FORM_PERSISTENT) {
         p.slots = reinterpret_cast<unsigned long long *>(ws + pl.off_slots);
         p.mail = &p.ctl->mail;
+        p.prune = pl.prune ? 1 : 0;
+        p.labels = reinterpret_cast<uint16_t *>(ws + pl.min_bytes);
     } else {
         p.block_sums = reinterpret_cast<float2 *>(ws + pl.off_bsum);
         p.seg_sums = reinterpret_cast<float2 *>(ws + pl.off_seg);

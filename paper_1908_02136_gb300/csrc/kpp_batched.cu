@@ -70,6 +70,7 @@ struct Wave {
     std::vector<std::vector<BatchEntry>> lists; // team jobs per CTA, in schedule order
     std::vector<int32_t> queue;                  // single-CTA jobs, longest first
     size_t nentries;
+    size_t smem; // dynamic shared memory of its CTAs
     size_t off_entries, off_first, off_queue, off_counter; // workspace offsets
 };
 
@@ -80,9 +81,16 @@ struct BatchPlan {
     std::vector<int64_t> chunk;
     std::vector<Wave> waves; // launched in this order
     // workspace layout
-    size_t off_jobs, off_ctls, off_slots, bytes;
+    size_t off_jobs, off_ctls, off_slots;
+    size_t min_bytes; // without the labels (such a workspace is accepted: every
+                      // pass then reads every row)
+    size_t off_labels, bytes;
     std::vector<size_t> slot_off; // per problem, relative to off_slots
+    std::vector<size_t> lab_off;  // per problem, relative to off_labels (kNoLabels: none)
 };
+
+constexpr int kBatchPruneMinK = 8; // fewer passes than this are all plain ones
+constexpr size_t kNoLabels = ~size_t(0);
 
 int elem_bytes(int dt) { return dt == KPP_F32 ? 4 : dt == KPP_BF16 ? 2 : 1; }
 
@@ -152,10 +160,19 @@ kpp_status make_batch_plan(const kpp_problem *pr, int32_t n, int dt, const kpp_o
         Wave w;
         w.d = d;
         w.fn = batched_fn(dt, d);
+        // rows of at least 16 bytes: passes skip rows (kpp_pass.cuh); the
+        // bounds' room follows the largest K of the wave
+        w.smem = 0;
+        if (d * eb >= 16.0)
+            for (int i : order)
+                w.smem = std::max(
+                    w.smem, (size_t)prune_layout(0, 0, pr[i].K, false, kPersistWarps).bytes);
         int resident = 0;
         if (!w.fn ||
+            cudaFuncSetAttribute((const void *)w.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)w.smem) != cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, (const void *)w.fn,
-                                                          kPersistThreads, 0) != cudaSuccess)
+                                                          kPersistThreads, w.smem) != cudaSuccess)
             return KPP_ERR_CUDA;
         if (resident < 1)
             return KPP_ERR_UNSUPPORTED;
@@ -231,7 +248,15 @@ kpp_status make_batch_plan(const kpp_problem *pr, int32_t n, int dt, const kpp_o
         soff += round_up(8 * 2 * kSlotWords * (size_t)bp->nblocks[i], 64);
     }
     off += round_up(soff, kAlign);
-    bp->bytes = off;
+    bp->min_bytes = bp->off_labels = off;
+    bp->lab_off.assign(n, kNoLabels);
+    size_t loff = 0;
+    for (int i = 0; i < n; ++i)
+        if (pr[i].d * eb >= 16.0 && pr[i].K >= kBatchPruneMinK) {
+            bp->lab_off[i] = loff;
+            loff += round_up(sizeof(uint16_t) * (size_t)pr[i].N, 64);
+        }
+    bp->bytes = off + round_up(loff, kAlign);
     return KPP_OK;
 }
 
@@ -261,8 +286,9 @@ kpp_status kpp_seed_batched(const kpp_problem *problems, int32_t n, kpp_dtype dt
     if (st != KPP_OK)
         return st;
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) % kAlign) != 0 ||
-        workspace_bytes < bp.bytes)
+        workspace_bytes < bp.min_bytes)
         return KPP_ERR_WORKSPACE;
+    const bool prune = workspace_bytes >= bp.bytes;
     char *ws = reinterpret_cast<char *>(workspace);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     // host image of the job table and the work lists
@@ -291,9 +317,13 @@ kpp_status kpp_seed_batched(const kpp_problem *problems, int32_t n, kpp_dtype dt
         p.nblocks = bp.nblocks[i];
         p.slots = reinterpret_cast<unsigned long long *>(ws + bp.off_slots + bp.slot_off[i]);
         p.exact_draws = (opts && opts->exact_draws) ? 1 : 0;
+        if (prune && bp.lab_off[i] != kNoLabels) {
+            p.prune = 1;
+            p.labels = reinterpret_cast<uint16_t *>(ws + bp.off_labels + bp.lab_off[i]);
+        }
         b.d = q.d;
     }
-    if (cudaMemsetAsync(ws, 0, bp.bytes, s) != cudaSuccess ||
+    if (cudaMemsetAsync(ws, 0, bp.min_bytes, s) != cudaSuccess ||
         cudaMemcpyAsync(ws + bp.off_jobs, jobs.data(), sizeof(BatchJob) * (size_t)n,
                         cudaMemcpyHostToDevice, s) != cudaSuccess)
         return KPP_ERR_CUDA;
@@ -337,7 +367,7 @@ kpp_status kpp_seed_batched(const kpp_problem *problems, int32_t n, kpp_dtype dt
         a.pa = pa;
         void *args[] = {&a};
         if (cudaLaunchCooperativeKernel((const void *)w.fn, dim3(bp.grid), dim3(kPersistThreads),
-                                        args, 0, s) != cudaSuccess)
+                                        args, w.smem, s) != cudaSuccess)
             return KPP_ERR_LAUNCH;
     }
     return KPP_OK;

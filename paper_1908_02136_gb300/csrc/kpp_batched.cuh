@@ -74,6 +74,7 @@ __device__ __forceinline__ void report(const Problem &p, const BatchArgs &a, int
 template <int DT, int D>
 __global__ void __launch_bounds__(kPersistThreads, 1) batched_kernel(BatchArgs a)
 {
+    extern __shared__ __align__(128) char smem[]; // the lists of the passes that skip rows
     __shared__ BlockShared sh;
     __shared__ int job_sh, rank_sh;
     const int list0 = a.first[blockIdx.x];
@@ -102,7 +103,7 @@ __global__ void __launch_bounds__(kPersistThreads, 1) batched_kernel(BatchArgs a
         if (j < 0)
             break;
         const Problem &p = a.jobs[j].p;
-        seed_blocks<DT, D, BatchGeom<DT, D>::L, D2_INPLACE>(p, a.pa, rank, nullptr, sh);
+        seed_blocks<DT, D, BatchGeom<DT, D>::L, D2_INPLACE, Geom<DT, D, 1>::WIDE>(p, a.pa, rank, smem, sh);
         report(p, a, rank);
     }
 }

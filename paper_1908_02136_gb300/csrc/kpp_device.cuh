@@ -80,6 +80,8 @@ struct Problem {
     unsigned long long *mail;  // persistent form: the drawn index, tagged with its pass
     int32_t recompute;         // streamed form: every pass rebuilds D^2 from all chosen seeds
     int32_t exact_draws;       // every draw decision in FP64 (the near-tie path), for testing
+    int32_t prune;             // persistent form: skip the rows that a pass cannot change
+    uint16_t *labels;          //   their nearest centres [N] (D^2 in the output array only)
     // point-sharded seeding (one contiguous row range of a larger problem):
     // the centre of the pass comes from the exchange buffer `xchg` (global
     // index, row scale, stored row), indices are global (< n_global), and a

@@ -46,6 +46,8 @@ struct PersistArgs {
 struct PersistentKernel {
     const void *fn_smem;   // D^2 in shared memory
     const void *fn_global; // D^2 in the output array
+    const void *prune_smem;   // the same with passes that skip rows, or null
+    const void *prune_global;
     int rows_align;          // rows per super-iteration; blocks are multiples of it
     int row_bytes;
     int lanes;
@@ -62,6 +64,10 @@ cudaError_t persistent_launch(const void *fn, int grid, size_t smem, const Probl
 // current device, if `asked` leaves every knob to the automatic choice.
 bool tuned_options(int64_t N, int32_t d, int32_t K, int dt, const kpp_options &asked,
                    kpp_options *out);
+
+// Whether kpp_seed's passes skip rows (kpp_pass.cuh) under this plan, given
+// kpp_workspace_size bytes of workspace.
+bool plan_skips_rows(int64_t N, int32_t d, int32_t K, kpp_dtype dtype, const kpp_options *opts);
 
 } // namespace kpp
 

@@ -169,6 +169,9 @@ struct PassIO {
     float2 *segs;          // segment sums of this CTA, one per warp (global or smem)
     uint64_t policy;       // L2 cache policy of global point loads (0: none)
     Control *ctl;          // status block (debug build: index checks report here)
+    uint16_t *lab;         // nearest centre of every row, indexed by row - r0 (shared
+                           //   memory for D2_SMEM, else global), or null
+    uint16_t lab_new;      // the label of this pass's centre
 };
 
 __device__ __forceinline__ uint4 ld_global_hint(const void *ptr, uint64_t policy)
@@ -267,6 +270,61 @@ __device__ __forceinline__ float update_d2(const PassIO &io, int64_t row, float 
     if (MODE == D2_SMEM && io.d2_out)
         io.d2_out[row] = v;
     return v;
+}
+
+// Squared distances of the rows of one batch (slots [jb, jb + JB) of a
+// 32-row group): each lane sums its slice of the rows, then the L lanes
+// sharing a row add up.  Lane l of a row group ends with slot l's sum in
+// `mine` once the batch holding that slot has been through.
+template <int DT, int D, int L_>
+__device__ __forceinline__ void batch_d2(const uint4 (&x)[Geom<DT, D, L_>::JB][Geom<DT, D, L_>::VPL],
+                                         const float (&sc)[Geom<DT, D, L_>::JB],
+                                         const CentreRegs<DT, D, L_> &cr, int jb, float &mine)
+{
+    using G = Geom<DT, D, L_>;
+    const int l = (threadIdx.x & 31) % G::L;
+    float part[G::JB];
+#pragma unroll
+    for (int q = 0; q < G::JB; ++q) {
+        float a0 = 0.f, a1 = 0.f;
+#pragma unroll
+        for (int v = 0; v < G::VPL; ++v) {
+            float f[G::EPV];
+            decode16<DT>(x[q][v], f);
+            cr.template accum<G::EPV>(f, v * G::EPV, sc[q], a0, a1);
+        }
+        part[q] = a0 + a1;
+    }
+    if constexpr (G::JB == G::L) {
+        // every slot of the row group is in this batch: reduce-scatter
+        // over the L lanes sharing the rows -- halving the live slots
+        // at each step, each lane keeping the half its bit selects --
+        // leaves slot l's sum on lane l.  Each lane adds the same
+        // partials in the same pairs as the butterfly below, so the
+        // sums are bit-identical to it, with log2(L) shuffle rounds
+        // for all L rows instead of log2(L) per row.
+#pragma unroll
+        for (int o = G::L / 2, n = G::JB; o > 0; o >>= 1, n >>= 1) {
+            const bool up = (l & o) != 0;
+#pragma unroll
+            for (int i = 0; i < n / 2; ++i) {
+                const float send = up ? part[i] : part[i + n / 2];
+                const float keep = up ? part[i + n / 2] : part[i];
+                part[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+        }
+        mine = part[0];
+    } else {
+#pragma unroll
+        for (int q = 0; q < G::JB; ++q) {
+            float sum = part[q];
+#pragma unroll
+            for (int o = G::L / 2; o > 0; o >>= 1)
+                sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            if (l == jb + q)
+                mine = sum;
+        }
+    }
 }
 
 // One pass over rows [r0, r1) by all warps of the CTA, each over its own
@@ -379,48 +437,7 @@ __device__ __forceinline__ Pair pass_rows(const PassIO &io, const CentreRegs<DT,
                     }
                 }
             }
-            float part[G::JB];
-#pragma unroll
-            for (int q = 0; q < G::JB; ++q) {
-                float a0 = 0.f, a1 = 0.f;
-#pragma unroll
-                for (int v = 0; v < G::VPL; ++v) {
-                    float f[G::EPV];
-                    decode16<DT>(x[q][v], f);
-                    cr.template accum<G::EPV>(f, v * G::EPV, sc[q], a0, a1);
-                }
-                part[q] = a0 + a1;
-            }
-            if constexpr (G::JB == G::L) {
-                // every slot of the row group is in this batch: reduce-scatter
-                // over the L lanes sharing the rows -- halving the live slots
-                // at each step, each lane keeping the half its bit selects --
-                // leaves slot l's sum on lane l.  Each lane adds the same
-                // partials in the same pairs as the butterfly below, so the
-                // sums are bit-identical to it, with log2(L) shuffle rounds
-                // for all L rows instead of log2(L) per row.
-#pragma unroll
-                for (int o = G::L / 2, n = G::JB; o > 0; o >>= 1, n >>= 1) {
-                    const bool up = (l & o) != 0;
-#pragma unroll
-                    for (int i = 0; i < n / 2; ++i) {
-                        const float send = up ? part[i] : part[i + n / 2];
-                        const float keep = up ? part[i + n / 2] : part[i];
-                        part[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-                    }
-                }
-                mine = part[0];
-            } else {
-#pragma unroll
-                for (int q = 0; q < G::JB; ++q) {
-                    float sum = part[q];
-#pragma unroll
-                    for (int o = G::L / 2; o > 0; o >>= 1)
-                        sum += __shfl_xor_sync(0xffffffffu, sum, o);
-                    if (l == jb + q)
-                        mine = sum;
-                }
-            }
+            batch_d2<DT, D, L_>(x, sc, cr, jb, mine);
             if (jb + G::JB == G::L) { // last batch of the super-iteration
                 const int64_t own_row = rb + (int64_t)l * (32 / G::L) + g;
                 if (own_row < seg_last)
@@ -520,6 +537,437 @@ __device__ __forceinline__ Pair pass_rows(const PassIO &io, const CentreRegs<DT,
     if (lane == 0)
         io.segs[warp] = make_float2(seg.hi, seg.lo);
     return seg;
+}
+
+// ---------------------------------------------------------------------------
+// Passes that read only the rows whose D^2 can still fall.
+//
+// Every row carries the label of its nearest chosen centre a.  For the new
+// centre c the triangle inequality gives |x - c| >= |c - a| - |x - a|, so a
+// row with 4 D^2 <= |c - a|^2 cannot come nearer (Elkan, "Using the triangle
+// inequality to accelerate k-means", ICML 2003; for the seeding, Raff, "Exact
+// acceleration of k-means++ and k-means||", IJCAI 2021).  The minimum keeps
+// its old value there, so leaving the row unread changes no bit of D^2.  The
+// computed squares carry a relative rounding of at most (d + 1) 2^-24 each
+// (d <= 4096: 2.5e-4); the test keeps a margin of 2^-8, several times their
+// sum.  Squares near the ends of the FP32 range (and NaN) skip nothing, or
+// only rows at D^2 = 0.
+//
+// The plain pass over a large set is bound by HBM, so the rows left out are
+// time saved: on mixtures with as many components as seeds a pass has to
+// read 34 % of the rows on average (99 % at the first seeds, under 1 % at the
+// last).  Whole seedings before and after: 10^7 x 64, K = 1024 FP32 381 -> 152
+// ms, BF16 225 -> 92 ms; 2 10^7 x 128, K = 2048 FP8 1337 -> 506 ms; 10^6 x 32,
+// K = 256 (in L2) 3.95 -> 3.55 ms; the 512-problem batch 40.6 -> 23.2 ms.  A
+// pass that reads every row costs 394 us here against 370 in the plain kernel
+// (10^7 x 64 FP32), 490 against 652 for FP8 (2 10^7 x 128).
+// ---------------------------------------------------------------------------
+constexpr int kPruneCentres = 2048; // centres with a bound; rows of later ones are always read
+constexpr uint16_t kNoLabel = 0xffff;
+
+// Largest D^2 of a row of centre a that centre c at squared distance s2 from
+// a cannot lower (negative: none).
+__device__ __forceinline__ float prune_bound(float s2)
+{
+    if (!(s2 < 1e37f))
+        return -1.f;
+    return s2 < 1e-30f ? 0.f : s2 * (0.25f * (1.f - 0x1.0p-8f));
+}
+
+// Largest number of rows read ahead of their arithmetic by a warp, and the
+// list of a warp's rows to read: those, one group short of complete and one
+// block of tested rows.
+constexpr int kPruneBlock = 8; // 32-row groups tested together
+constexpr int kPruneAhead = 128;
+constexpr int kPruneList = 512;
+static_assert(kPruneList >= kPruneAhead + 32 + 32 + 32 * kPruneBlock, "the list holds them");
+constexpr int kPruneRing = 8192; // bytes a warp reads ahead
+
+// 16- and 4-byte asynchronous copies from global to shared memory.
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
+__device__ __forceinline__ void cp_async4(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+
+__device__ __forceinline__ void cp_async_commit()
+{
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+template <int N> __device__ __forceinline__ void cp_async_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// The squared distances of a list of rows to the centre, by one warp, with
+// the row groups and the arithmetic of pass_rows (bit-identical results).
+// The rows in flight sit in a ring in shared memory instead of registers:
+// 8 KB a warp, 128 KB an SM, which is what the plain pass keeps in flight (a
+// register ring beside the list's state spills).  Every lane copies, waits
+// for and reads its own 16-byte vectors, so the ring needs no barrier.  The
+// list grows by whole groups of 32 items; the last one is padded with rows
+// that may be read (n says how many items count).
+//   row_at(i, k)     offset in rows from `base` of item i + k (i a multiple of
+//                    32 plus the lane's row group, k a constant below 32)
+//   pre(own)         what sink wants of the lane's own item, loaded early
+//   sink(own, v, p)  called on the lane that owns the item
+template <int DT, int D, int L_, class RowAt, class Pre, class Sink> struct RowPipe {
+    using G = Geom<DT, D, L_>;
+    static_assert(G::WIDE, "rows of at least 16 bytes");
+    static constexpr int JB0 = G::VPL >= 4 ? 1 : 4 / G::VPL;
+    static constexpr int JB = JB0 < G::L ? JB0 : G::L; // slots per batch
+    static constexpr int NB = G::L / JB;               // batches per group
+    static constexpr int BR = JB * (32 / G::L);        // rows per batch
+    static constexpr int BB = JB * G::VPL * 512;       // bytes per batch
+    static constexpr int R0 = kPruneRing / BB < kPruneAhead / BR ? kPruneRing / BB : kPruneAhead / BR;
+    static constexpr int R = R0 < 2 ? 2 : R0; // batches in flight
+    static_assert(R * BB <= kPruneRing && (R & (R - 1)) == 0, "the ring holds them");
+
+    const CentreRegs<DT, D, L_> &cr;
+    const char *src0;     // this lane's first vector of row 0 of the list's base
+    const float *scales0; // its FP8 scale
+    uint32_t ring, sring; // this lane's first vector; the FP8 scales of the rows in flight
+    RowAt row_at;
+    Pre pre;
+    Sink sink;
+    int n = 0;        // items of the list so far
+    int groups = 0;   // issued
+    uint32_t it = 0;  // batches issued
+    int done = 0;     // groups consumed
+    float part[G::L]; // this lane's share of each slot's row
+
+    __device__ __forceinline__ RowPipe(const PassIO &io, int64_t base,
+                                       const CentreRegs<DT, D, L_> &cr_, char *ring_, RowAt r, Pre p,
+                                       Sink s)
+        : cr(cr_), row_at(r), pre(p), sink(s)
+    {
+        const int lane = threadIdx.x & 31;
+        src0 = io.gpts + base * G::RB + (lane % G::L) * 16;
+        scales0 = DT == KPP_FP8_E4M3 ? io.scales + base : nullptr;
+        const uint32_t r0 = (uint32_t)__cvta_generic_to_shared(ring_);
+        ring = r0 + lane * 16;
+        sring = r0 + kPruneRing;
+    }
+
+    // offsets of the rows of batch jb of the next group
+    __device__ __forceinline__ void rows_of(int jb, uint32_t (&row)[JB]) const
+    {
+        const int g = (threadIdx.x & 31) / G::L;
+#pragma unroll
+        for (int q = 0; q < JB; ++q)
+            row[q] = row_at(groups * 32 + g, (jb * JB + q) * (32 / G::L));
+    }
+
+    __device__ __forceinline__ void issue(int jb, const uint32_t (&row)[JB])
+    {
+        const uint32_t slot = it & (R - 1);
+        const uint32_t dst = ring + slot * BB;
+#pragma unroll
+        for (int q = 0; q < JB; ++q) {
+            const char *src = src0 + (uint64_t)row[q] * G::RB;
+#pragma unroll
+            for (int v = 0; v < G::VPL; ++v)
+                cp_async16(dst + (q * G::VPL + v) * 512, src + v * G::L * 16);
+        }
+        if constexpr (DT == KPP_FP8_E4M3) {
+            const int lane = threadIdx.x & 31;
+            if (BR == 32 || lane < BR)
+                cp_async4(sring + (slot * BR + lane) * 4,
+                          scales0 + row_at(groups * 32 + lane, jb * BR));
+        }
+        cp_async_commit();
+        ++it;
+    }
+
+    // the batch issued `back` batches ago
+    __device__ __forceinline__ void consume(int jb, uint32_t back)
+    {
+        const int lane = threadIdx.x & 31, g = lane / G::L, l = lane % G::L;
+        if (DT == KPP_FP8_E4M3)
+            __syncwarp(); // the scales were copied by other lanes
+        const uint32_t slot = (it - back) & (R - 1);
+        const uint32_t src = ring + slot * BB;
+        const int own = done * 32 + l * (32 / G::L) + g;
+        decltype(pre(0)) mine{};
+        if (jb == NB - 1)
+            mine = pre(own);
+        float sum[JB];
+#pragma unroll
+        for (int q = 0; q < JB; ++q) {
+            float s = 1.0f;
+            if constexpr (DT == KPP_FP8_E4M3)
+                asm volatile("ld.shared.f32 %0, [%1];"
+                             : "=f"(s)
+                             : "r"(sring + (slot * BR + q * (32 / G::L) + g) * 4));
+            float a0 = 0.f, a1 = 0.f;
+#pragma unroll
+            for (int v = 0; v < G::VPL; ++v) {
+                uint4 x;
+                asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                             : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w)
+                             : "r"(src + (q * G::VPL + v) * 512));
+                float f[G::EPV];
+                decode16<DT>(x, f);
+                cr.template accum<G::EPV>(f, v * G::EPV, s, a0, a1);
+            }
+            sum[q] = a0 + a1;
+        }
+#pragma unroll
+        for (int q = 0; q < JB; ++q)
+            part[jb * JB + q] = sum[q];
+        if (DT == KPP_FP8_E4M3)
+            __syncwarp(); // the scales are read before their slot is filled again
+        if (jb == NB - 1) {
+            // reduce-scatter as in pass_rows: the same pairs, slot l's sum on lane l
+#pragma unroll
+            for (int o = G::L / 2, w = G::L; o > 0; o >>= 1, w >>= 1) {
+                const bool up = (l & o) != 0;
+#pragma unroll
+                for (int i = 0; i < w / 2; ++i) {
+                    const float send = up ? part[i] : part[i + w / 2];
+                    const float keep = up ? part[i + w / 2] : part[i];
+                    part[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                }
+            }
+            if (own < n)
+                sink(own, part[0], mine);
+            ++done;
+        }
+    }
+
+    // reads the next group of 32 items; the oldest batches in flight make room
+    __device__ __forceinline__ void group()
+    {
+#pragma unroll
+        for (int jb = 0; jb < NB; ++jb) {
+            uint32_t row[JB];
+            rows_of(jb, row); // before the wait: off the batch's critical path
+            if (it >= (uint32_t)R) {
+                cp_async_wait<R - 1>();
+                consume((jb + NB * R - R) % NB, R);
+            }
+            issue(jb, row);
+        }
+        ++groups;
+    }
+
+    // the batches still in flight
+    __device__ __forceinline__ void drain()
+    {
+        cp_async_wait<0>();
+        int left = it < (uint32_t)R ? (int)it : R; // the oldest is batch (it - left) % NB of its group
+        while (left > 0) {
+#pragma unroll
+            for (int b = 0; b < NB; ++b)
+                if (left > 0 && (it - left) % NB == (uint32_t)b) {
+                    consume(b, left);
+                    --left;
+                }
+        }
+    }
+
+    __device__ __forceinline__ bool full() const { return n - groups * 32 >= 32; }
+    __device__ __forceinline__ bool rest() const { return n > groups * 32; }
+};
+
+template <int DT, int D, int L_, class RowAt, class Pre, class Sink>
+__device__ __forceinline__ RowPipe<DT, D, L_, RowAt, Pre, Sink>
+make_row_pipe(const PassIO &io, int64_t base, const CentreRegs<DT, D, L_> &cr, char *ring, RowAt r,
+              Pre p, Sink s)
+{
+    return RowPipe<DT, D, L_, RowAt, Pre, Sink>(io, base, cr, ring, r, p, s);
+}
+
+// A row's new D^2 with its previous one given; stores what changed.
+template <int MODE>
+__device__ __forceinline__ float keep_nearest(const PassIO &io, int64_t row, float v, float old)
+{
+    if (!io.first && !(v < old))
+        return old;
+    if (MODE == D2_INPLACE)
+        io.d2[row] = v;
+    else
+        io.d2s[row - io.r0] = v;
+    if (io.lab)
+        io.lab[row - io.r0] = io.lab_new;
+    return v;
+}
+
+// Shared memory of the passes that skip rows, beside the block's D^2 and
+// chunk sums (byte offsets from `base`): labels (D^2 in shared memory only),
+// the bounds and rows of the chosen centres, every warp's ring (with room for
+// FP8 scales) and list of rows to read, and (D^2 in the output array only)
+// the D^2 of those rows.
+struct PruneLayout {
+    int64_t lab, thr, cidx, ring, list, list_d2, bytes;
+};
+// (a ring starts on a 128-byte boundary: at 16 bytes past one every 32-byte
+// sector lands in two of shared memory and is requested from L2 twice --
+// 20.7 GB crossed to the SMs for 10.2 GB of points)
+constexpr int kPruneRingBytes = kPruneRing + 4 * kPruneAhead;
+static_assert(kPruneRingBytes % 128 == 0, "rings are 128-byte aligned");
+
+template <int MODE> struct ListRow {
+    using type = uint32_t;
+};
+template <> struct ListRow<D2_SMEM> {
+    using type = uint16_t; // offsets in a block that fits shared memory
+};
+
+__host__ __device__ __forceinline__ PruneLayout prune_layout(int64_t base, int64_t chunk, int K,
+                                                             bool d2_in_smem, int nwarps)
+{
+    PruneLayout p;
+    const int64_t kp = K < kPruneCentres ? K : kPruneCentres;
+    p.lab = (base + 15) & ~15ll;
+    p.thr = p.lab + (d2_in_smem ? ((2 * chunk + 15) & ~15ll) : 0);
+    p.cidx = p.thr + 4 * kp;
+    p.ring = (p.cidx + 4 * kp + 127) & ~127ll;
+    p.list = p.ring + (int64_t)kPruneRingBytes * nwarps;
+    p.list_d2 = p.list + (d2_in_smem ? 2ll : 4ll) * kPruneList * nwarps;
+    p.bytes = p.list_d2 + (d2_in_smem ? 0 : 4ll * kPruneList * nwarps);
+    return p;
+}
+
+struct PruneIO {
+    int64_t ci;          // the new centre's row
+    float *thr;          // room for the bounds of the chosen centres (shared memory)
+    const int32_t *cidx; // their rows (shared memory)
+    int nc;              // chosen centres to take a bound for (0: read every row)
+    char *ring;          // this warp's ring (shared)
+    void *list;          // this warp's list of rows to read (shared)
+    float *list_d2;      // their D^2 (D2_INPLACE; shared)
+    int *active;         // out: rows each warp read (shared)
+};
+
+// The pass over this warp's segment that reads only the rows whose D^2 can
+// fall (all of them when pr.nc is 0).  A block of 32-row groups at a time:
+// their D^2 and labels (the next block's loads are in flight meanwhile) are
+// tested one row per lane, and the rows left go to the warp's list, which
+// feeds the row pipe a full group at a time, so the reads of one block's rows
+// are in flight while the next are tested.  A skipped row costs 6 bytes, most
+// of them from L2, in place of its own.
+template <int DT, int D, int L_, int MODE>
+__device__ __forceinline__ void pass_rows_pruned(const PassIO &io, const PruneIO &pr)
+{
+    using G = Geom<DT, D, L_>;
+    using Row = typename ListRow<MODE>::type;
+    constexpr int U = kPruneBlock;
+    const int lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
+    const int nwarps = blockDim.x >> 5;
+    int64_t seg_first, seg_last;
+    segment_rows(io.r0, io.r1 - io.r0, G::SW, nwarps, warp, &seg_first, &seg_last);
+    const int rows = (int)(seg_last - seg_first); // offsets in the segment are ints
+    const int64_t rel = seg_first - io.r0;
+    CentreRegs<DT, D, L_> cr;
+    cr.load(io.gpts, io.scales, pr.ci);
+    if (pr.nc > 0) {
+        // the distance of the new centre to every chosen one, each warp a
+        // share of them
+        const int per = (pr.nc + nwarps - 1) / nwarps;
+        const int f = warp * per;
+        const int n = pr.nc - f < per ? pr.nc - f : per;
+        if (n > 0) {
+            auto pipe = make_row_pipe<DT, D, L_>(
+                io, 0, cr, pr.ring,
+                [&](int i, int k) { return (uint32_t)pr.cidx[f + (i + k < n ? i + k : n - 1)]; },
+                [](int) { return 0; }, [&](int i, float v, int) { pr.thr[f + i] = prune_bound(v); });
+            pipe.n = n;
+            while (pipe.rest())
+                pipe.group();
+            pipe.drain();
+        }
+        __syncthreads();
+    }
+    Row *list = reinterpret_cast<Row *>(pr.list);
+    float *list_d2 = pr.list_d2;
+    Pair lacc{};
+    struct Own {
+        int row;
+        float d2;
+    };
+    auto pipe = make_row_pipe<DT, D, L_>(
+        io, seg_first, cr, pr.ring,
+        [&](int i, int k) { return (uint32_t)list[i % kPruneList + k]; },
+        [&](int i) {
+            Own o;
+            o.row = (int)list[i % kPruneList];
+            o.d2 = MODE == D2_INPLACE ? list_d2[i % kPruneList] : io.d2s[rel + o.row];
+            return o;
+        },
+        [&](int, float v, const Own &o) {
+            if (kpp_check(io.ctl, seg_first + o.row < seg_last, 111))
+                lacc.add(keep_nearest<MODE>(io, seg_first + o.row, v, o.d2));
+        });
+    const int nblock = (rows + 32 * U - 1) / (32 * U);
+    float d2[U];
+    uint16_t lb[U];
+    auto load = [&](int j) { // (in pass 0 both are still unset, and every row is read)
+        const int b = (io.reverse ? nblock - 1 - j : j) * 32 * U;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int o = b + 32 * u + lane;
+            const bool in = o < rows && kpp_check(io.ctl, seg_first + o < io.r1, 110);
+            if (MODE == D2_SMEM) {
+                d2[u] = in ? io.d2s[rel + o] : 0.f;
+                lb[u] = in ? io.lab[rel + o] : 0;
+            } else {
+                d2[u] = in ? __ldcg(io.d2 + seg_first + o) : 0.f;
+                lb[u] = in && pr.nc > 0 ? __ldcg(io.lab + rel + o) : 0;
+            }
+        }
+    };
+    if (nblock > 0)
+        load(0);
+    for (int j = 0; j < nblock; ++j) {
+        const int b = (io.reverse ? nblock - 1 - j : j) * 32 * U;
+        int n = pipe.n;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int o = b + 32 * u + lane;
+            const float t = lb[u] < pr.nc ? pr.thr[lb[u]] : -1.f;
+            const bool must = o < rows && (io.first || !(d2[u] <= t));
+            const unsigned m = __ballot_sync(0xffffffffu, must);
+            if (must) {
+                const int at = (n + __popc(m & ((1u << lane) - 1u))) % kPruneList;
+                list[at] = (Row)o;
+                if (MODE == D2_INPLACE)
+                    list_d2[at] = d2[u];
+            }
+            n += __popc(m);
+            lacc.add(must ? 0.f : d2[u]);
+        }
+        pipe.n = n;
+        if (j + 1 < nblock) {
+            load(j + 1);
+        } else { // the last group's other items: rows that may be read
+            list[(n + lane) % kPruneList] = 0;
+            if (MODE == D2_INPLACE)
+                list_d2[(n + lane) % kPruneList] = 0.f;
+        }
+        __syncwarp(); // the list is read by other lanes
+        while (pipe.full())
+            pipe.group();
+    }
+    if (pipe.rest())
+        pipe.group();
+    pipe.drain();
+    if (MODE == D2_SMEM && io.d2_out) {
+        __syncwarp(); // the rows' last stores came from other lanes
+        for (int o = lane; o < rows; o += 32)
+            io.d2_out[seg_first + o] = io.d2s[rel + o];
+    }
+    const Pair seg = warp_pair_sum(lacc);
+    if (lane == 0) {
+        io.segs[warp] = make_float2(seg.hi, seg.lo);
+        pr.active[warp] = pipe.n;
+    }
 }
 
 // The CTA's D^2 sum: warp pairs added in warp order, rounded once to FP64.

@@ -27,6 +27,8 @@ bool persistent_lookup(int dt, int d, int lanes, PersistentKernel *out)
         return false;
     out->fn_smem = reinterpret_cast<const void *>(best->fn_smem);
     out->fn_global = reinterpret_cast<const void *>(best->fn_global);
+    out->prune_smem = reinterpret_cast<const void *>(best->prune_smem);
+    out->prune_global = reinterpret_cast<const void *>(best->prune_global);
     out->rows_align = best->sw;
     out->row_bytes = best->rb;
     out->lanes = best->lanes;

@@ -8,7 +8,9 @@
 // super-iterations of every warp's segment are copied into shared memory in
 // pass 0 and read from there afterwards; the rest are streamed from HBM/L2
 // each pass, in alternating directions and with an L2 evict-last policy so
-// that what the previous pass left in L2 is read first.
+// that what the previous pass left in L2 is read first.  Built with PRUNE, the
+// kernel has no point cache and its passes skip the rows that the new centre
+// cannot bring nearer (kpp_pass.cuh).
 //
 // Between passes there is no counter barrier.  Each CTA publishes its block
 // sum as one tagged 64-bit word; waiting for all nblocks words of the pass is
@@ -53,7 +55,15 @@ struct DrawShared {
 struct BlockShared {
     float2 segsum[kPersistWarps];
     DrawShared ds;
+    int active[kPersistWarps]; // rows each warp read in the last pass that skipped rows
+    int few;                   // they were few enough to go on skipping
 };
+
+// Passes test for rows to skip while at most kPruneKeep of the block's rows
+// had to be read; above that they read every row -- no bounds to compute, which
+// cost up to 10 us at 1000 centres -- and every kPruneProbe-th pass tests again.
+constexpr float kPruneKeep = 0.8f;
+constexpr int kPruneProbe = 8;
 
 // The seeding of problem p by a team of p.nblocks co-resident CTAs, this CTA
 // being member b: p.slots and p.mail are the team's own exchange words.
@@ -61,7 +71,9 @@ struct BlockShared {
 // unused when a.cache_supers == 0 and MODE == D2_INPLACE).  Returns when the
 // seeding is done, or early -- the same way on every member -- on an error
 // recorded in the status word.
-template <int DT, int D, int L, int MODE>
+// PRUNE: built with the passes that skip rows (p.prune turns them on); without
+// it the kernel is the plain one, its pass inline.
+template <int DT, int D, int L, int MODE, bool PRUNE>
 __device__ __forceinline__ void seed_blocks(const Problem &p, const PersistArgs &a, const int b,
                                             char *smem, BlockShared &sh)
 {
@@ -80,6 +92,20 @@ __device__ __forceinline__ void seed_blocks(const Problem &p, const PersistArgs 
     const bool chunk_path = (MODE == D2_SMEM) && (p.chunk + 31) / 32 <= kMaxChunks;
     const uint64_t policy =
         a.l2_hint == 1 ? policy_evict_last() : (a.l2_hint == 2 ? policy_evict_first() : 0ull);
+
+    // passes that skip rows: labels, bounds and lists behind the chunk sums
+    // (the plan leaves no point cache beside them)
+    const bool can_prune = PRUNE && p.prune;
+    PruneLayout pl{};
+    if (PRUNE)
+        pl = prune_layout(MODE == D2_SMEM
+                              ? ((4 * p.chunk + 15) & ~15ll) + 8 * ((p.chunk + 31) / 32)
+                              : 0,
+                          p.chunk, p.K, MODE == D2_SMEM, kPersistWarps);
+    float *thr = reinterpret_cast<float *>(smem + pl.thr);
+    int32_t *cidx = reinterpret_cast<int32_t *>(smem + pl.cidx);
+    if (threadIdx.x == 0)
+        sh.few = 0;
 
     // the plan's limits: this block exists, the level-1 stage and the chunk
     // sums hold what the draw will put there (every CTA sees the same values)
@@ -104,8 +130,6 @@ __device__ __forceinline__ void seed_blocks(const Problem &p, const PersistArgs 
     for (int m = 0; m < p.K; ++m) {
         const bool last = (m == p.K - 1);
         const int next = m + 1;
-        CentreRegs<DT, D, L> cr;
-        cr.load(p.points, p.scales, ci);
 
         PassIO io{};
         io.ctl = p.ctl;
@@ -123,7 +147,31 @@ __device__ __forceinline__ void seed_blocks(const Problem &p, const PersistArgs 
         io.d2s = d2s;
         io.segs = segsum;
         io.policy = policy;
-        pass_rows<DT, D, L, MODE>(io, cr);
+        bool prune = false;
+        if constexpr (PRUNE) {
+            if (can_prune) {
+                io.lab = MODE == D2_SMEM ? reinterpret_cast<uint16_t *>(smem + pl.lab)
+                                         : p.labels + r0;
+                io.lab_new = m < kPruneCentres ? (uint16_t)m : kNoLabel;
+                prune = m > 0 && (sh.few || m % kPruneProbe == 1);
+                if (threadIdx.x == 0 && m < kPruneCentres)
+                    cidx[m] = (int32_t)ci; // read from the next pass on
+            }
+            PruneIO pr;
+            pr.ci = ci;
+            pr.thr = thr;
+            pr.cidx = cidx;
+            pr.nc = !prune ? 0 : (m < kPruneCentres ? m : kPruneCentres);
+            pr.ring = smem + pl.ring + warp * kPruneRingBytes;
+            pr.list = smem + pl.list + warp * kPruneList * (int)sizeof(typename ListRow<MODE>::type);
+            pr.list_d2 = reinterpret_cast<float *>(smem + pl.list_d2) + warp * kPruneList;
+            pr.active = sh.active;
+            pass_rows_pruned<DT, D, L, MODE>(io, pr);
+        } else {
+            CentreRegs<DT, D, L> cr;
+            cr.load(p.points, p.scales, ci);
+            pass_rows<DT, D, L, MODE>(io, cr);
+        }
         __syncthreads();
 
         // publish this block's pair sum (segments in warp order)
@@ -186,6 +234,12 @@ __device__ __forceinline__ void seed_blocks(const Problem &p, const PersistArgs 
                 ds.th[(next + 1) & 1] =
                     thresh_for_u(philox_uniform(p.seed, p.stream_id, (uint64_t)(next + 1)),
                                  p.exact_draws);
+            if (threadIdx.x == 64 && prune) {
+                int read = 0;
+                for (int w = 0; w < kPersistWarps; ++w)
+                    read += sh.active[w];
+                sh.few = (float)read <= kPruneKeep * (float)(r1 - r0);
+            }
             if (chunk_path && !forced) {
                 for (int c = threadIdx.x - 32; c < nchunks; c += blockDim.x - 32) {
                     const int64_t rb = r0 + 32ll * c;
@@ -338,13 +392,13 @@ __device__ __forceinline__ void seed_blocks(const Problem &p, const PersistArgs 
     }
 }
 
-template <int DT, int D, int L, int MODE>
+template <int DT, int D, int L, int MODE, bool PRUNE>
 __global__ void __launch_bounds__(kPersistThreads, 1)
     persistent_kernel(Problem p, PersistArgs a)
 {
-    extern __shared__ __align__(16) char smem[];
+    extern __shared__ __align__(128) char smem[];
     __shared__ BlockShared sh;
-    seed_blocks<DT, D, L, MODE>(p, a, blockIdx.x, smem, sh);
+    seed_blocks<DT, D, L, MODE, PRUNE>(p, a, blockIdx.x, smem, sh);
 }
 
 // One specialisation of the persistent kernel, as listed by the per-dtype
@@ -354,18 +408,22 @@ using PersistFn = void (*)(Problem, PersistArgs);
 struct PSpec {
     int dt, d, lanes, sw, rb;
     PersistFn fn_smem, fn_global;
+    PersistFn prune_smem, prune_global; // with passes that skip rows; null for narrow rows
 };
 
 template <int DT, int D, int L>
 constexpr PSpec make_pspec()
 {
-    return PSpec{DT,
-                 D,
-                 Geom<DT, D, L>::L,
-                 Geom<DT, D, L>::SW,
-                 Geom<DT, D, L>::RB,
-                 &persistent_kernel<DT, D, L, D2_SMEM>,
-                 &persistent_kernel<DT, D, L, D2_INPLACE>};
+    using G = Geom<DT, D, L>;
+    PSpec s{DT,   D,       G::L,
+            G::SW, G::RB,   &persistent_kernel<DT, D, L, D2_SMEM, false>,
+            &persistent_kernel<DT, D, L, D2_INPLACE, false>,
+            nullptr, nullptr};
+    if constexpr (G::WIDE) {
+        s.prune_smem = &persistent_kernel<DT, D, L, D2_SMEM, true>;
+        s.prune_global = &persistent_kernel<DT, D, L, D2_INPLACE, true>;
+    }
+    return s;
 }
 
 // The specialisations built for each stored type (one translation unit each,
