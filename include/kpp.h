@@ -350,8 +350,10 @@ KPP_API void kpp_tune_clear(void);
  *   centres_out [K x d] FP32: the means (may not alias `centres`)
  *   counts_out  [K] int64 or NULL: points per centre
  *   phi_out     [1] FP64 or NULL: sum of d2 (the cost of the assignment)
- *   workspace   >= kpp_lloyd_workspace_size(N, d, K) bytes, 256-byte aligned,
- *               prepared once by kpp_lloyd_prepare for these points
+ *   workspace   kpp_lloyd_workspace_size(N, d, K) bytes, 256-byte aligned,
+ *               prepared once by kpp_lloyd_prepare for these points (without
+ *               its last part, 4 N bytes and more for the points' order by
+ *               label, the update still runs, more slowly)
  * The assignment runs on the tensor cores: |c|^2 - 2 x.c with x and c split
  * into two BF16 planes (hi + lo) and x.c = hi.hi + hi.lo + lo.hi accumulated
  * in FP32, so a label can differ from the exact nearest centre only when two

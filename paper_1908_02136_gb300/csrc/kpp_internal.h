@@ -81,6 +81,9 @@ kpp_status lloyd_assign_device_count(const float *centres, const long long *row0
                                      int32_t *labels_out, void *workspace, size_t workspace_bytes,
                                      cudaStream_t stream);
 
+// Workspace of kpp_lloyd_prepare and the assignments alone (0 if invalid).
+size_t lloyd_assign_workspace(int64_t N, int32_t d, int32_t K);
+
 cudaError_t quantize_bf16(const float *x, int64_t n, uint16_t *out, cudaStream_t stream);
 cudaError_t quantize_fp8(const float *x, int64_t N, int d, uint8_t *q, float *scales,
                          cudaStream_t stream);

@@ -106,7 +106,7 @@ Layout layout(int64_t N, int32_t d, int64_t cand_cap)
     L.off_ct = off = round_up(off, kAlign);
     off += (size_t)L.ldc * d * 4;
     L.off_lloyd = off = round_up(off, kAlign);
-    L.lloyd_bytes = kpp_lloyd_workspace_size(N, d, lloyd_k(N));
+    L.lloyd_bytes = lloyd_assign_workspace(N, d, lloyd_k(N));
     off += L.lloyd_bytes;
     L.bytes = round_up(off, kAlign);
     return L;

@@ -55,9 +55,22 @@ size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 struct Layout {
     int dp;   // padded feature count (64 or 128)
-    int grid; // CTAs of the per-point kernels
-    size_t off_phi, off_plo, off_chi, off_clo, off_cn, off_sums, off_counts, off_partial, bytes;
+    int grid; // most CTAs of the update kernels
+    size_t off_phi, off_plo, off_chi, off_clo, off_cn, off_sums, off_counts, off_partial;
+    size_t min_bytes; // without the update's point order (accepted: the direct update runs)
+    size_t off_perm, off_start, off_ticket, off_base, bytes;
 };
+
+// CTAs of the kernels that order the points by label: a point range each.
+constexpr int kOrdThreads = 512;
+constexpr int kOrdMaxCtas = 608;
+constexpr int kOrdPoints = 4096; // smallest range
+
+int ord_ctas(int64_t N)
+{
+    const int64_t n = (N + kOrdPoints - 1) / kOrdPoints;
+    return (int)(n < kOrdMaxCtas ? n : kOrdMaxCtas);
+}
 
 bool shape_ok(int64_t N, int32_t d, int32_t K)
 {
@@ -87,6 +100,15 @@ Layout layout(int64_t N, int32_t d, int32_t K)
     off += (size_t)K * 8;
     L.off_partial = off = round_up(off, kAlign);
     off += (size_t)L.grid * 8;
+    L.min_bytes = off = round_up(off, kAlign);
+    L.off_perm = off;
+    off += (size_t)N * 4;
+    L.off_start = off = round_up(off, kAlign);
+    off += ((size_t)K + 1) * 4;
+    L.off_ticket = off = round_up(off, kAlign);
+    off += kAlign;
+    L.off_base = off;
+    off += (size_t)ord_ctas(N) * K * 4;
     L.bytes = round_up(off, kAlign);
     return L;
 }
@@ -102,24 +124,29 @@ __device__ __forceinline__ void split_bf16(float v, __nv_bfloat16 &hi, __nv_bflo
 
 // A thread per (row, group of 8 features): eight FP32 loads, one 16-byte
 // store per plane.  dp / 8 is 8 or 16, so the indexing is shifts and masks.
+__device__ __forceinline__ void split_group(const float *x, int64_t g, int d, int dp, int sh,
+                                            __nv_bfloat16 *hi, __nv_bfloat16 *lo)
+{
+    const int64_t r = g >> sh;
+    const int j0 = (int)(g & ((1 << sh) - 1)) << 3;
+    __align__(16) __nv_bfloat16 h[8], l[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const int j = j0 + u;
+        split_bf16(j < d ? x[r * d + j] : 0.f, h[u], l[u]);
+    }
+    *reinterpret_cast<uint4 *>(hi + r * dp + j0) = *reinterpret_cast<const uint4 *>(h);
+    *reinterpret_cast<uint4 *>(lo + r * dp + j0) = *reinterpret_cast<const uint4 *>(l);
+}
+
 __device__ __forceinline__ void split_rows_body(const float *x, int64_t rows, int d, int dp,
                                                 __nv_bfloat16 *hi, __nv_bfloat16 *lo)
 {
     const int sh = dp == 64 ? 3 : 4;
     const int64_t n = rows << sh;
     for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n;
-         g += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = g >> sh;
-        const int j0 = (int)(g & ((1 << sh) - 1)) << 3;
-        __align__(16) __nv_bfloat16 h[8], l[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int j = j0 + u;
-            split_bf16(j < d ? x[r * d + j] : 0.f, h[u], l[u]);
-        }
-        *reinterpret_cast<uint4 *>(hi + r * dp + j0) = *reinterpret_cast<const uint4 *>(h);
-        *reinterpret_cast<uint4 *>(lo + r * dp + j0) = *reinterpret_cast<const uint4 *>(l);
-    }
+         g += (int64_t)gridDim.x * blockDim.x)
+        split_group(x, g, d, dp, sh, hi, lo);
 }
 
 __global__ void split_rows_kernel(const float *x, int64_t rows, int d, int dp, __nv_bfloat16 *hi,
@@ -128,37 +155,54 @@ __global__ void split_rows_kernel(const float *x, int64_t rows, int d, int dp, _
     split_rows_body(x, rows, d, dp, hi, lo);
 }
 
-// The same for rows [*row0, *row0 + *rows) of `base`, counts read on the device.
-__global__ void split_rows_dev_kernel(const float *base, const long long *row0,
-                                      const int32_t *rows, int d, int dp, __nv_bfloat16 *hi,
-                                      __nv_bfloat16 *lo)
-{
-    split_rows_body(base + *row0 * d, *rows, d, dp, hi, lo);
-}
+// What the assignment needs of the centres, in one launch: their BF16 planes
+// (the first `split_ctas` CTAs), |c_k|^2 in FP32 (a thread per centre, the
+// CTAs after them) and, by all of them, the cleared control block and
+// `nzero` cleared words.  With row0 and rows set the centres are rows
+// [*row0, *row0 + *rows) of `base`, counts read on the device.  Three
+// launches and two memsets before: 8 us of a 10^6-point step.
+struct CentreArgs {
+    const float *base;
+    const long long *row0; // or null: the first row
+    const int32_t *rows;   // or null: K rows
+    int32_t K, d, dp;
+    int32_t split_ctas;
+    __nv_bfloat16 *hi, *lo;
+    float *cn;
+    Control *ctl;
+    uint32_t *zero;
+    int64_t nzero;
+};
 
-// |c_k|^2 in FP32 (one thread per centre); the device-count form reads K and
-// the first row from device memory.
-__device__ __forceinline__ void centre_norm(const float *c, int k, int d, float *cn)
-{
-    float s = 0.f;
-    for (int j = 0; j < d; ++j)
-        s = fmaf(c[(int64_t)k * d + j], c[(int64_t)k * d + j], s);
-    cn[k] = s;
-}
+constexpr int kCentreThreads = 128;
 
-__global__ void centre_norms_kernel(const float *c, int K, int d, float *cn)
+__global__ void __launch_bounds__(kCentreThreads) centres_kernel(CentreArgs a)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < K)
-        centre_norm(c, k, d, cn);
-}
-
-__global__ void centre_norms_dev_kernel(const float *base, const long long *row0,
-                                        const int32_t *K, int d, float *cn)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < *K)
-        centre_norm(base + *row0 * d, k, d, cn);
+    const float *c = a.row0 ? a.base + *a.row0 * a.d : a.base;
+    const int K = a.rows ? *a.rows : a.K;
+    const int t = threadIdx.x;
+    if (blockIdx.x == 0 && t < (int)(sizeof(Control) / 4))
+        reinterpret_cast<uint32_t *>(a.ctl)[t] = 0u;
+    for (int64_t i = blockIdx.x * (int64_t)kCentreThreads + t; i < a.nzero;
+         i += (int64_t)gridDim.x * kCentreThreads)
+        a.zero[i] = 0u;
+    if ((int)blockIdx.x >= a.split_ctas) {
+        const int k = ((int)blockIdx.x - a.split_ctas) * kCentreThreads + t;
+        if (k < K) {
+            // features in order (the scores' rounding follows from it)
+            const float *row = c + (int64_t)k * a.d;
+            float s = 0.f;
+#pragma unroll 8
+            for (int j = 0; j < a.d; ++j)
+                s = fmaf(row[j], row[j], s);
+            a.cn[k] = s;
+        }
+        return;
+    }
+    const int sh = a.dp == 64 ? 3 : 4;
+    const int64_t g = blockIdx.x * (int64_t)kCentreThreads + t; // (row, group of 8 features)
+    if (g < ((int64_t)K << sh))
+        split_group(c, g, a.d, a.dp, sh, a.hi, a.lo);
 }
 
 // ---------------------------------------------------------------------------
@@ -917,11 +961,310 @@ UpdateFn update_fn(int d)
     return &lloyd_update_kernel<4, 8>;
 }
 
-__global__ void lloyd_finalize_kernel(const float *c_in, int K, int d, const double *sums,
-                                      const unsigned long long *counts, float *c_out,
-                                      int64_t *counts_out, const double *partial, int nparts,
-                                      double *phi_out)
+// ---------------------------------------------------------------------------
+// The update over points ordered by label.
+//
+// With the points of a centre next to each other, a warp sums a run of rows
+// in registers: no shared-memory atomic per point and feature, and the
+// centre's features are loaded once per run.  The direct kernel above spends
+// 106 warp instructions a point (ncu: issue and shared-memory latency, DRAM
+// 19 % busy); here about 17 remain and the walk is bound by the random reads
+// of whole rows.  A counting sort makes the order: counts per label and
+// range, the label starts, then every point's position -- 20 bytes a point of
+// L2 traffic.  10^7 x 64, K = 1024: update 0.65 ms in place of 1.88
+// (0.56 of it the walk, 4.6 TB/s); 10^6 x 32, K = 256: about 60 us in place of 111.
+// ---------------------------------------------------------------------------
+
+// A point's label; one that an assignment which gave up on a wait left unset
+// (the status says so) counts as 0.
+__device__ __forceinline__ int32_t label_at(const int32_t *labels, int64_t i, int K)
 {
+    const int32_t l = __ldg(labels + i);
+    return (unsigned)l < (unsigned)K ? l : 0;
+}
+
+// Counts of every label in each CTA's range of points.  base[cta][k] gets the
+// number of label-k points of the CTAs that reserved before it (any order:
+// only the sums' grouping depends on it); the CTA that finishes last turns
+// the totals into starts.
+__global__ void __launch_bounds__(kOrdThreads)
+    lloyd_count_kernel(const int32_t *labels, int64_t N, int K, unsigned long long *counts,
+                       int32_t *base, int32_t *start, unsigned *ticket)
+{
+    extern __shared__ int s_cnt[]; // [K]
+    __shared__ int wsum[kOrdThreads / 32];
+    __shared__ int is_last;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    for (int k = t; k < K; k += kOrdThreads)
+        s_cnt[k] = 0;
+    __syncthreads();
+    const int64_t per = (N + gridDim.x - 1) / gridDim.x;
+    const int64_t lo = blockIdx.x * per, hi = lo + per < N ? lo + per : N;
+    for (int64_t i0 = lo + t; i0 < hi; i0 += 4 * kOrdThreads) {
+        int32_t l[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            l[u] = i0 + u * kOrdThreads < hi ? label_at(labels, i0 + u * kOrdThreads, K) : -1;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (l[u] >= 0)
+                atomicAdd(s_cnt + l[u], 1);
+    }
+    __syncthreads();
+    int32_t *b = base + (int64_t)blockIdx.x * K;
+    for (int k = t; k < K; k += kOrdThreads)
+        if (s_cnt[k])
+            b[k] = (int32_t)atomicAdd(counts + k, (unsigned long long)s_cnt[k]);
+    __threadfence();
+    __syncthreads();
+    if (t == 0)
+        is_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!is_last)
+        return;
+    __threadfence();
+    // exclusive scan of the totals: a run of labels per thread
+    const int run = (K + kOrdThreads - 1) / kOrdThreads;
+    const int k0 = t * run < K ? t * run : K, k1 = k0 + run < K ? k0 + run : K;
+    int own = 0;
+    for (int k = k0; k < k1; ++k)
+        own += (int)__ldcg(counts + k);
+    int inc = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o)
+            inc += y;
+    }
+    if (lane == 31)
+        wsum[warp] = inc;
+    __syncthreads();
+    int at = inc - own;
+    for (int w = 0; w < warp; ++w)
+        at += wsum[w];
+    for (int k = k0; k < k1; ++k) {
+        start[k] = at;
+        at += (int)__ldcg(counts + k);
+    }
+    if (t == 0)
+        start[K] = (int32_t)N;
+}
+
+// perm[position] = point, positions grouped by label.
+__global__ void __launch_bounds__(kOrdThreads)
+    lloyd_order_kernel(const int32_t *labels, int64_t N, int K, const int32_t *base,
+                       const int32_t *start, int32_t *perm)
+{
+    extern __shared__ int s_at[]; // [K] next position of this range's points
+    const int t = threadIdx.x;
+    const int32_t *b = base + (int64_t)blockIdx.x * K;
+    for (int k = t; k < K; k += kOrdThreads)
+        s_at[k] = start[k] + b[k]; // (b[k] is not set where the range has no such point)
+    __syncthreads();
+    const int64_t per = (N + gridDim.x - 1) / gridDim.x;
+    const int64_t lo = blockIdx.x * per, hi = lo + per < N ? lo + per : N;
+    for (int64_t i0 = lo + t; i0 < hi; i0 += 4 * kOrdThreads) {
+        int32_t l[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            l[u] = i0 + u * kOrdThreads < hi ? label_at(labels, i0 + u * kOrdThreads, K) : -1;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (l[u] >= 0)
+                perm[atomicAdd(s_at + l[u], 1)] = (int32_t)(i0 + u * kOrdThreads);
+    }
+}
+
+constexpr int kSegThreads = 256;
+constexpr int kSegCtas = 3; // per SM
+
+// Every warp takes a contiguous range of positions and walks it run by run
+// (a run: positions of one label).  LD lanes share a row (32 / LD rows a
+// step), lane j of them holding features j, j + LD, ...; ROWS steps are in
+// flight.  A batch's rows are summed in FP32 per lane and added to an FP32
+// two-sum pair, a run's pairs go to the FP64 totals with one atomic a feature.
+// D^2 is the FP32 difference form, its lane partials added over the row's
+// lanes.
+template <int LD, int VEC, int ROWS>
+__global__ void __launch_bounds__(kSegThreads, kSegCtas)
+    lloyd_segment_kernel(const float *__restrict__ x, int64_t N, int d, int K,
+                         const float *__restrict__ c, const int32_t *__restrict__ perm,
+                         const int32_t *__restrict__ start, float *d2_out, double *sums,
+                         double *partial)
+{
+    constexpr int RPS = 32 / LD; // rows per step
+    extern __shared__ int s_start[]; // [K + 1]
+    __shared__ float2 wsum[kSegThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int sub = lane / LD, j = lane % LD;
+    for (int k = threadIdx.x; k <= K; k += kSegThreads)
+        s_start[k] = start[k];
+    __syncthreads();
+    const int64_t nw = (int64_t)gridDim.x * (kSegThreads / 32);
+    const int64_t per = (N + nw - 1) / nw;
+    int64_t p = ((int64_t)blockIdx.x * (kSegThreads / 32) + warp) * per;
+    const int64_t p1 = p + per < N ? p + per : N;
+    Pair mine{}; // the cost of the points this lane reports
+    if (p < p1) {
+        int k = 0, kh = K - 1; // the label of position p: the first k with start[k + 1] > p
+        while (k < kh) {
+            const int m = (k + kh) >> 1;
+            if (s_start[m + 1] > p)
+                kh = m;
+            else
+                k = m + 1;
+        }
+        for (; p < p1; ++k) {
+            const int64_t e = s_start[k + 1] < p1 ? s_start[k + 1] : p1;
+            if (e <= p)
+                continue; // no point
+            float cv[VEC], hi[VEC], lo[VEC];
+#pragma unroll
+            for (int t = 0; t < VEC; ++t) {
+                const int f = j + LD * t;
+                cv[t] = f < d ? c[(int64_t)k * d + f] : 0.f;
+                hi[t] = lo[t] = 0.f;
+            }
+            for (; p < e; p += ROWS * RPS) {
+                int32_t row[ROWS];
+#pragma unroll
+                for (int q = 0; q < ROWS; ++q) {
+                    const int64_t at = p + q * RPS + sub;
+                    row[q] = at < e ? perm[at] : -1;
+                }
+                float xv[ROWS][VEC];
+#pragma unroll
+                for (int q = 0; q < ROWS; ++q)
+#pragma unroll
+                    for (int t = 0; t < VEC; ++t) {
+                        const int f = j + LD * t;
+                        xv[q][t] = row[q] >= 0 && f < d ? x[(int64_t)row[q] * d + f] : 0.f;
+                    }
+                float part[ROWS], acc[VEC];
+#pragma unroll
+                for (int t = 0; t < VEC; ++t)
+                    acc[t] = 0.f;
+#pragma unroll
+                for (int q = 0; q < ROWS; ++q) {
+                    float s = 0.f;
+#pragma unroll
+                    for (int t = 0; t < VEC; ++t) {
+                        const float u = xv[q][t] - cv[t];
+                        s = fmaf(u, u, s);
+                        acc[t] += xv[q][t];
+                    }
+                    part[q] = s;
+                }
+#pragma unroll
+                for (int t = 0; t < VEC; ++t) {
+                    Pair h{hi[t], lo[t]};
+                    h.add(acc[t]);
+                    hi[t] = h.hi;
+                    lo[t] = h.lo;
+                }
+                if constexpr (LD == 32) {
+                    // reduce-scatter: row q's sum ends in lane q * 32 / ROWS
+#pragma unroll
+                    for (int m = 16, w = ROWS / 2; w >= 1; m >>= 1, w >>= 1) {
+                        const bool up = (lane & m) != 0;
+#pragma unroll
+                        for (int i = 0; i < w; ++i) {
+                            const float send = up ? part[i] : part[i + w];
+                            const float keep = up ? part[i + w] : part[i];
+                            part[i] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+                        }
+                    }
+#pragma unroll
+                    for (int o = 16 / ROWS; o >= 1; o >>= 1)
+                        part[0] += __shfl_xor_sync(0xffffffffu, part[0], o);
+                    constexpr int SH = 32 / ROWS;
+                    const int q = lane / SH;
+                    if (lane % SH == 0 && p + q < e) {
+                        if (d2_out)
+                            d2_out[perm[p + q]] = part[0];
+                        mine.add(part[0]);
+                    }
+                } else {
+#pragma unroll
+                    for (int q = 0; q < ROWS; ++q) {
+#pragma unroll
+                        for (int o = LD / 2; o >= 1; o >>= 1)
+                            part[q] += __shfl_xor_sync(0xffffffffu, part[q], o);
+                        if (j == 0 && row[q] >= 0) {
+                            if (d2_out)
+                                d2_out[row[q]] = part[q];
+                            mine.add(part[q]);
+                        }
+                    }
+                }
+            }
+            p = e;
+#pragma unroll
+            for (int t = 0; t < VEC; ++t) {
+                double v = (double)hi[t] + (double)lo[t];
+#pragma unroll
+                for (int o = LD; o < 32; o <<= 1)
+                    v += __shfl_xor_sync(0xffffffffu, v, o);
+                const int f = j + LD * t;
+                if (sub == 0 && f < d)
+                    atomicAdd(sums + (int64_t)k * d + f, v);
+            }
+        }
+    }
+    const Pair wt = warp_pair_sum(mine);
+    if (lane == 0)
+        wsum[warp] = make_float2(wt.hi, wt.lo);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        Pair t{};
+        for (int w = 0; w < kSegThreads / 32; ++w)
+            t.add(Pair{wsum[w].x, wsum[w].y});
+        partial[blockIdx.x] = (double)t.hi + (double)t.lo;
+    }
+}
+
+// Which update: ordering the points costs two launches and 20 bytes a point
+// against the direct kernel's work per point and feature (and its walk over
+// the points once per tile of centres).  Whole steps measured, ordered against
+// direct: 120 000 x 2 49 / 49 us, x 32 56 / 56, x 100 76 / 82; 500 000 x 2
+// 94 / 123, x 64 (K = 64) 109 / 134; 30 000 x 100 51 / 41; over many tiles
+// 8 000 x 128 (K = 2000) 84 / 95, 30 000 97 / 123.
+bool update_ordered(int64_t N, int d, int K)
+{
+    const int tiles = (K + update_tile(K, d) - 1) / update_tile(K, d);
+    return N >= 200000 || N * d >= 10000000 || (tiles >= 3 && N * d >= 1000000);
+}
+
+using SegmentFn = void (*)(const float *, int64_t, int, int, const float *, const int32_t *,
+                           const int32_t *, float *, double *, double *);
+
+// Lanes per row by d, so that few lanes idle; 64 rows' worth of loads or 8 KB
+// a warp in flight.
+SegmentFn segment_fn(int d)
+{
+    if (d <= 4)
+        return &lloyd_segment_kernel<4, 1, 16>;
+    if (d <= 8)
+        return &lloyd_segment_kernel<8, 1, 16>;
+    if (d <= 16)
+        return &lloyd_segment_kernel<16, 1, 16>;
+    if (d <= 32)
+        return &lloyd_segment_kernel<32, 1, 16>;
+    if (d <= 64)
+        return &lloyd_segment_kernel<32, 2, 16>;
+    if (d <= 96)
+        return &lloyd_segment_kernel<32, 3, 8>;
+    return &lloyd_segment_kernel<32, 4, 8>;
+}
+
+constexpr int kFinThreads = 256;
+
+__global__ void __launch_bounds__(kFinThreads)
+    lloyd_finalize_kernel(const float *c_in, int K, int d, const double *sums,
+                          const unsigned long long *counts, float *c_out, int64_t *counts_out,
+                          const double *partial, int nparts, double *phi_out)
+{
+    __shared__ double sh[kFinThreads / 32];
     const int64_t n = (int64_t)K * d;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
          e += (int64_t)gridDim.x * blockDim.x) {
@@ -932,11 +1275,15 @@ __global__ void lloyd_finalize_kernel(const float *c_in, int K, int d, const dou
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; counts_out && k < K;
          k += gridDim.x * blockDim.x)
         counts_out[k] = (int64_t)counts[k];
-    if (blockIdx.x == 0 && threadIdx.x == 0 && phi_out) {
+    // phi by the last CTA: a share of the partials per thread, then a tree (one
+    // thread adding them all took 11 us: an FP64 add is 64 cycles)
+    if (blockIdx.x == gridDim.x - 1 && phi_out) {
         double s = 0.0;
-        for (int b = 0; b < nparts; ++b)
+        for (int b = threadIdx.x; b < nparts; b += kFinThreads)
             s += partial[b];
-        *phi_out = s;
+        s = block_sum<kFinThreads>(s, sh);
+        if (threadIdx.x == 0)
+            *phi_out = s;
     }
 }
 
@@ -1037,16 +1384,18 @@ int sm_count()
     return sms;
 }
 
-// The assignment of N prepared points to K centres.  With row0 and kdev set,
+// The assignment of N prepared points to K centres; `nzero` words at `zero`
+// are cleared on the way.  With row0 and kdev set,
 // the centres are rows [*row0, *row0 + *kdev) of `centres` and K is only the
 // largest count the launch is sized for; both are read on the device.
 kpp_status assign_impl(const float *centres, const long long *row0, const int32_t *kdev, int32_t K,
                        int64_t N, int32_t d, int32_t *labels_out, void *workspace,
-                       size_t workspace_bytes, cudaStream_t s)
+                       size_t workspace_bytes, cudaStream_t s, uint32_t *zero = nullptr,
+                       int64_t nzero = 0)
 {
     const Layout L = layout(N, d, K);
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) % kAlign) != 0 ||
-        workspace_bytes < L.bytes)
+        workspace_bytes < L.min_bytes)
         return KPP_ERR_WORKSPACE;
     char *ws = reinterpret_cast<char *>(workspace);
     const int sms = sm_count();
@@ -1079,17 +1428,22 @@ kpp_status assign_impl(const float *centres, const long long *row0, const int32_
     a.timeout_ns = 2000000000ull;
     if (a.stages < 2)
         return KPP_ERR_UNSUPPORTED;
-    if (cudaMemsetAsync(ws, 0, sizeof(Control), s) != cudaSuccess)
-        return KPP_ERR_CUDA;
-    if (kdev) {
-        split_rows_dev_kernel<<<(K * L.dp / 8 + 255) / 256, 256, 0, s>>>(centres, row0, kdev, d,
-                                                                         L.dp, chi, clo);
-        centre_norms_dev_kernel<<<(K + 127) / 128, 128, 0, s>>>(centres, row0, kdev, d, cn);
-    } else {
-        split_rows_kernel<<<(K * L.dp / 8 + 255) / 256, 256, 0, s>>>(centres, K, d, L.dp, chi,
-                                                                     clo);
-        centre_norms_kernel<<<(K + 127) / 128, 128, 0, s>>>(centres, K, d, cn);
-    }
+    CentreArgs ca;
+    ca.base = centres;
+    ca.row0 = kdev ? row0 : nullptr;
+    ca.rows = kdev;
+    ca.K = K;
+    ca.d = d;
+    ca.dp = L.dp;
+    ca.split_ctas = (int)(((int64_t)K * L.dp / 8 + kCentreThreads - 1) / kCentreThreads);
+    ca.hi = chi;
+    ca.lo = clo;
+    ca.cn = cn;
+    ca.ctl = a.ctl;
+    ca.zero = zero;
+    ca.nzero = nzero;
+    centres_kernel<<<ca.split_ctas + (K + kCentreThreads - 1) / kCentreThreads, kCentreThreads, 0,
+                     s>>>(ca);
     if (use_pair_form()) {
         // CTA pairs: persistent, as many clusters of two as fit at once
         AssignArgs a2 = a;
@@ -1135,6 +1489,11 @@ kpp_status assign_impl(const float *centres, const long long *row0, const int32_
 
 } // namespace
 
+size_t lloyd_assign_workspace(int64_t N, int32_t d, int32_t K)
+{
+    return shape_ok(N, d, K) ? layout(N, d, K).min_bytes : 0;
+}
+
 kpp_status lloyd_assign_device_count(const float *centres, const long long *row0,
                                      const int32_t *kdev, int32_t kmax, int64_t N, int32_t d,
                                      int32_t *labels_out, void *workspace, size_t workspace_bytes,
@@ -1166,7 +1525,7 @@ kpp_status kpp_lloyd_prepare(const float *points, int64_t N, int32_t d, int32_t 
         return KPP_ERR_INVALID_ARG;
     const Layout L = layout(N, d, K);
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) % kAlign) != 0 ||
-        workspace_bytes < L.bytes)
+        workspace_bytes < L.min_bytes)
         return KPP_ERR_WORKSPACE;
     char *ws = reinterpret_cast<char *>(workspace);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
@@ -1198,7 +1557,7 @@ kpp_status kpp_lloyd_step(const float *points, int64_t N, int32_t d, const float
         return KPP_ERR_INVALID_ARG;
     const Layout L = layout(N, d, K);
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) % kAlign) != 0 ||
-        workspace_bytes < L.bytes)
+        workspace_bytes < L.min_bytes)
         return KPP_ERR_WORKSPACE;
     char *ws = reinterpret_cast<char *>(workspace);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
@@ -1208,23 +1567,43 @@ kpp_status kpp_lloyd_step(const float *points, int64_t N, int32_t d, const float
     double *sums = reinterpret_cast<double *>(ws + L.off_sums);
     auto *counts = reinterpret_cast<unsigned long long *>(ws + L.off_counts);
     double *partial = reinterpret_cast<double *>(ws + L.off_partial);
+    const bool ordered = workspace_bytes >= L.bytes && update_ordered(N, d, K);
     const size_t usmem = (size_t)update_tile(K, d) * ((size_t)d * 4 + 4);
     const UpdateFn ufn = update_fn(d);
-    if (cudaFuncSetAttribute(ufn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)usmem) !=
-        cudaSuccess)
+    if (!ordered && cudaFuncSetAttribute(ufn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)usmem) != cudaSuccess)
         return KPP_ERR_CUDA;
+    auto *ticket = reinterpret_cast<unsigned *>(ws + L.off_ticket);
+    if (ordered && cudaMemsetAsync(ticket, 0, sizeof(unsigned), s) != cudaSuccess)
+        return KPP_ERR_CUDA;
+    // (the sums and counts are cleared by the assignment's first kernel)
     const kpp_status st =
-        kpp_lloyd_assign(centres, N, d, K, labels_out, workspace, workspace_bytes, stream);
+        assign_impl(centres, nullptr, nullptr, K, N, d, labels_out, workspace, workspace_bytes, s,
+                    reinterpret_cast<uint32_t *>(sums), (int64_t)((L.off_partial - L.off_sums) / 4));
     if (st != KPP_OK)
         return st;
-    if (cudaMemsetAsync(ws + L.off_sums, 0, L.off_partial - L.off_sums, s) != cudaSuccess)
-        return KPP_ERR_CUDA;
-    const int ugrid = sms < L.grid ? sms : L.grid;
-    ufn<<<ugrid, kUpdThreads, usmem, s>>>(points, N, d, K, centres, labels_out, d2_out, sums,
-                                          counts, partial);
-    lloyd_finalize_kernel<<<(K * d + 255) / 256, 256, 0, s>>>(centres, K, d, sums, counts,
-                                                              centres_out, counts_out, partial,
-                                                              ugrid, phi_out);
+    int parts;
+    if (ordered) {
+        int32_t *perm = reinterpret_cast<int32_t *>(ws + L.off_perm);
+        int32_t *start = reinterpret_cast<int32_t *>(ws + L.off_start);
+        int32_t *base = reinterpret_cast<int32_t *>(ws + L.off_base);
+        const int octas = ord_ctas(N);
+        const size_t osmem = (size_t)K * 4;
+        lloyd_count_kernel<<<octas, kOrdThreads, osmem, s>>>(labels_out, N, K, counts, base, start,
+                                                             ticket);
+        lloyd_order_kernel<<<octas, kOrdThreads, osmem, s>>>(labels_out, N, K, base, start, perm);
+        // a full wave; fewer CTAs where a warp would get less than two batches
+        const int64_t most = (N + 32 * (kSegThreads / 32) - 1) / (32 * (kSegThreads / 32));
+        parts = (int)(most < kSegCtas * sms ? most : kSegCtas * sms);
+        segment_fn(d)<<<parts, kSegThreads, osmem + 4, s>>>(points, N, d, K, centres, perm, start,
+                                                            d2_out, sums, partial);
+    } else {
+        parts = sms < L.grid ? sms : L.grid;
+        ufn<<<parts, kUpdThreads, usmem, s>>>(points, N, d, K, centres, labels_out, d2_out, sums,
+                                              counts, partial);
+    }
+    lloyd_finalize_kernel<<<(K * d + kFinThreads - 1) / kFinThreads, kFinThreads, 0, s>>>(
+        centres, K, d, sums, counts, centres_out, counts_out, partial, parts, phi_out);
     return cudaGetLastError() == cudaSuccess ? KPP_OK : KPP_ERR_LAUNCH;
 }
 
