@@ -213,6 +213,8 @@ struct AssignArgs {
     int32_t K;
     const int32_t *Kdev; // if set, K is read here (written by an earlier launch)
     int32_t nk;     // feature chunks (dp / 64)
+    int32_t ksteps; // 16-feature MMA steps that hold features, ceil(d / 16): the padding's
+                    // zeros add nothing (10^6 x 32, K = 256: half the MMAs)
     int32_t stages; // centre-tile stages in shared memory
     int32_t abufs;  // point-tile buffers (2: the next group's load overlaps this one)
     const float *cn;
@@ -618,10 +620,18 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     if (warp == 0 && lane == 0) {
         // ---- producer (both CTAs): own point tile, own half of each centre tile ----
-        uint32_t it = 0, g = 0;
-        for (int64_t gp = cl0; gp < n_grp && !abort_flag; gp += ncl, ++it) {
-            const uint32_t ab = it % a.abufs, ause = it / a.abufs;
-            if (ause > 0 && !mbar_wait_cluster(&a_empty[ab], (ause - 1) & 1, a.timeout_ns)) {
+        // Stages and point buffers are counted round with their phase, here
+        // and in the MMA issuer: the one thread that issues the MMAs sets
+        // their pace at d <= 64 (12 MMAs of 128 cycles a tile), so its
+        // divisions by run-time counts, a timer read before every wait and a
+        // descriptor built per MMA cost the tensor pipe time.  Without them
+        // 10^7 points x 64, K = 1024 2.79 -> 2.61 ms, 4 10^6 x 128, K = 2048
+        // 3.51 -> 3.31; with the padding's MMAs left out (a.ksteps) 10^6 x 32,
+        // K = 256 104 -> 89 us.
+        uint32_t ab = 0, aph = 0, s = 0, ph = 0;
+        bool a_used = false, b_used = false; // every buffer / stage has been filled once
+        for (int64_t gp = cl0; gp < n_grp && !abort_flag; gp += ncl) {
+            if (a_used && !mbar_wait_cluster(&a_empty[ab], aph ^ 1, a.timeout_ns)) {
                 fail(a.ctl, &abort_flag);
                 break;
             }
@@ -634,9 +644,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 tma_load_2d_pair(a_tile(ab, 1, k), &map_plo, fa, k * kBK, y);
             }
             for (int ct = 0; ct < n_ct && !abort_flag; ++ct) {
-                for (int k = 0; k < a.nk; ++k, ++g) {
-                    const uint32_t s = g % NS, use = g / NS;
-                    if (use > 0 && !mbar_wait_cluster(&b_empty[s], (use - 1) & 1, a.timeout_ns)) {
+                for (int k = 0; k < a.nk; ++k) {
+                    if (b_used && !mbar_wait_cluster(&b_empty[s], ph ^ 1, a.timeout_ns)) {
                         fail(a.ctl, &abort_flag);
                         break;
                     }
@@ -646,7 +655,17 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const int yc = ct * kPN + (int)rank * kPNH;
                     tma_load_2d_pair(sB + (s * 2 + 0) * kBBytes, &map_chi, fb, k * kBK, yc);
                     tma_load_2d_pair(sB + (s * 2 + 1) * kBBytes, &map_clo, fb, k * kBK, yc);
+                    if (++s == (uint32_t)NS) {
+                        s = 0;
+                        ph ^= 1;
+                        b_used = true;
+                    }
                 }
+            }
+            if (++ab == (uint32_t)a.abufs) {
+                ab = 0;
+                aph ^= 1;
+                a_used = true;
             }
         }
         if (abort_flag) {
@@ -659,11 +678,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     } else if (warp == 1 && lane == 0 && rank == 0) {
         // ---- MMA issuer (even CTA) ----
         const uint32_t idesc = idesc_bf16_f32(2 * kBM, kPN);
-        uint32_t it = 0, g = 0, t = 0;
+        uint32_t ab = 0, aph = 0, s = 0, ph = 0, t = 0;
         bool issued = false;
-        for (int64_t gp = cl0; gp < n_grp && !abort_flag; gp += ncl, ++it) {
-            const uint32_t ab = it % a.abufs, ause = it / a.abufs;
-            if (!mbar_wait_cluster(&a_full[ab], ause & 1, a.timeout_ns)) {
+        for (int64_t gp = cl0; gp < n_grp && !abort_flag; gp += ncl) {
+            if (!mbar_wait_cluster(&a_full[ab], aph, a.timeout_ns)) {
                 fail(a.ctl, &abort_flag);
                 break;
             }
@@ -677,29 +695,39 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
                 fence_after_sync();
                 const uint32_t d_tmem = tmem + buf * kPN;
-                for (int k = 0; k < a.nk; ++k, ++g) {
-                    const uint32_t s = g % NS, use = g / NS;
-                    if (!mbar_wait_cluster(&b_full[s], use & 1, a.timeout_ns)) {
+                for (int k = 0; k < a.nk; ++k) {
+                    if (!mbar_wait_cluster(&b_full[s], ph, a.timeout_ns)) {
                         fail(a.ctl, &abort_flag);
                         break;
                     }
                     fence_after_sync();
-                    const uint32_t bh = smem_u32(sB + (s * 2 + 0) * kBBytes);
-                    const uint32_t bl = smem_u32(sB + (s * 2 + 1) * kBBytes);
-                    const uint32_t ah = smem_u32(a_tile(ab, 0, k));
-                    const uint32_t al = smem_u32(a_tile(ab, 1, k));
-#pragma unroll
-                    for (int kk = 0; kk < kBK / 16; ++kk) {
-                        const uint32_t o = kk * 32;
-                        mma_bf16_pair(d_tmem, sdesc_k_sw128(ah + o), sdesc_k_sw128(bh + o), idesc,
+                    // descriptors advance by 32 bytes (2 units) per 16 features
+                    const uint64_t dah = sdesc_k_sw128(smem_u32(a_tile(ab, 0, k)));
+                    const uint64_t dal = sdesc_k_sw128(smem_u32(a_tile(ab, 1, k)));
+                    const uint64_t dbh = sdesc_k_sw128(smem_u32(sB + (s * 2 + 0) * kBBytes));
+                    const uint64_t dbl = sdesc_k_sw128(smem_u32(sB + (s * 2 + 1) * kBBytes));
+                    auto step = [&](int kk) {
+                        mma_bf16_pair(d_tmem, dah + 2 * kk, dbh + 2 * kk, idesc,
                                       (k | kk) ? 1u : 0u);
-                        mma_bf16_pair(d_tmem, sdesc_k_sw128(ah + o), sdesc_k_sw128(bl + o), idesc,
-                                      1u);
-                        mma_bf16_pair(d_tmem, sdesc_k_sw128(al + o), sdesc_k_sw128(bh + o), idesc,
-                                      1u);
+                        mma_bf16_pair(d_tmem, dah + 2 * kk, dbl + 2 * kk, idesc, 1u);
+                        mma_bf16_pair(d_tmem, dal + 2 * kk, dbh + 2 * kk, idesc, 1u);
+                    };
+                    const int steps = a.ksteps - k * (kBK / 16); // that hold features
+                    if (steps >= kBK / 16) {
+#pragma unroll
+                        for (int kk = 0; kk < kBK / 16; ++kk)
+                            step(kk);
+                    } else {
+#pragma unroll 1
+                        for (int kk = 0; kk < steps; ++kk)
+                            step(kk);
                     }
                     issued = true;
                     mma_commit_pair(&b_empty[s], 0x3); // both halves of stage s are free
+                    if (++s == (uint32_t)NS) {
+                        s = 0;
+                        ph ^= 1;
+                    }
                 }
                 if (abort_flag)
                     break;
@@ -708,6 +736,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (abort_flag)
                 break;
             mma_commit_pair(&a_empty[ab], 0x3);
+            if (++ab == (uint32_t)a.abufs) {
+                ab = 0;
+                aph ^= 1;
+            }
         }
         if (issued) { // every MMA issued completes before the pair frees its tensor memory
             mma_commit_pair(&done, 0x1);
@@ -1420,6 +1452,7 @@ kpp_status assign_impl(const float *centres, const long long *row0, const int32_
     a.K = K;
     a.Kdev = kdev;
     a.nk = nk;
+    a.ksteps = (d + 15) / 16;
     a.abufs = assign_abufs(nk, K);
     a.stages = assign_stages(nk, K, a.abufs);
     a.cn = cn;

@@ -46,17 +46,23 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *b)
 }
 // Waits for the phase of parity `parity` to complete.  Gives up (false)
 // after `timeout_ns` nanoseconds.
+__device__ __forceinline__ bool mbar_try(uint64_t *b, uint32_t parity)
+{
+    uint32_t done;
+    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+                 " selp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(done)
+                 : "r"(smem_u32(b)), "r"(parity)
+                 : "memory");
+    return done != 0;
+}
 __device__ __forceinline__ bool mbar_wait(uint64_t *b, uint32_t parity, uint64_t timeout_ns)
 {
+    if (mbar_try(b, parity)) // the timer is read only by waits that wait
+        return true;
     const uint64_t t0 = gtimer();
     for (uint32_t i = 1;; ++i) {
-        uint32_t done;
-        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-                     " selp.u32 %0, 1, 0, p;\n}\n"
-                     : "=r"(done)
-                     : "r"(smem_u32(b)), "r"(parity)
-                     : "memory");
-        if (done)
+        if (mbar_try(b, parity))
             return true;
         if ((i & 63u) == 0 && gtimer() - t0 > timeout_ns)
             return false;
@@ -233,17 +239,23 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t caddr)
 }
 // mbar_wait with cluster-scope acquire: for barriers that other CTAs of the
 // cluster (or their copies and MMAs) complete.
+__device__ __forceinline__ bool mbar_try_cluster(uint64_t *b, uint32_t parity)
+{
+    uint32_t done;
+    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, "
+                 "[%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(done)
+                 : "r"(smem_u32(b)), "r"(parity)
+                 : "memory");
+    return done != 0;
+}
 __device__ __forceinline__ bool mbar_wait_cluster(uint64_t *b, uint32_t parity, uint64_t timeout_ns)
 {
+    if (mbar_try_cluster(b, parity))
+        return true;
     const uint64_t t0 = gtimer();
     for (uint32_t i = 1;; ++i) {
-        uint32_t done;
-        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, "
-                     "[%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-                     : "=r"(done)
-                     : "r"(smem_u32(b)), "r"(parity)
-                     : "memory");
-        if (done)
+        if (mbar_try_cluster(b, parity))
             return true;
         if ((i & 63u) == 0 && gtimer() - t0 > timeout_ns)
             return false;
