@@ -103,8 +103,8 @@ kpp_status plan_streamed(int64_t N, int32_t d, int dt, const kpp_options &o, int
     return KPP_OK;
 }
 
-kpp_status plan_persistent_at(int64_t N, int32_t K, const kpp_options &o, int sms, int per_sm,
-                              Plan *pl);
+kpp_status plan_persistent_at(int64_t N, int32_t d, int32_t K, int dt, const kpp_options &o, int sms,
+                              int per_sm, Plan *pl);
 
 // The small form: one CTA, if the points and D^2 fit its shared memory.
 kpp_status plan_small(int64_t N, int32_t d, int dt, Plan *pl)
@@ -139,26 +139,26 @@ kpp_status plan_small(int64_t N, int32_t d, int dt, Plan *pl)
 }
 
 // The persistent plan at the requested CTAs per SM, or fewer if that many
-// cannot be co-resident.
+// cannot be co-resident.  any_d: also for a d without a specialisation.
 kpp_status plan_persistent(int64_t N, int32_t d, int32_t K, int dt, const kpp_options &o, int sms,
-                           Plan *pl)
+                           bool any_d, Plan *pl)
 {
-    if (!persistent_lookup(dt, d, o.lanes_per_row, &pl->pk))
+    if (!persistent_lookup(dt, d, o.lanes_per_row, any_d, &pl->pk))
         return KPP_ERR_UNSUPPORTED;
     int per_sm = o.ctas_per_sm > 0 ? o.ctas_per_sm : 1;
     if (per_sm > 4)
         return KPP_ERR_INVALID_ARG;
     kpp_status st = KPP_ERR_UNSUPPORTED;
     for (; per_sm >= 1; --per_sm) {
-        st = plan_persistent_at(N, K, o, sms, per_sm, pl);
+        st = plan_persistent_at(N, d, K, dt, o, sms, per_sm, pl);
         if (st != KPP_ERR_UNSUPPORTED)
             return st;
     }
     return st;
 }
 
-kpp_status plan_persistent_at(int64_t N, int32_t K, const kpp_options &o, int sms, int per_sm,
-                              Plan *pl)
+kpp_status plan_persistent_at(int64_t N, int32_t d, int32_t K, int dt, const kpp_options &o, int sms,
+                              int per_sm, Plan *pl)
 {
     int dev = 0, coop = 0, optin = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -169,7 +169,14 @@ kpp_status plan_persistent_at(int64_t N, int32_t K, const kpp_options &o, int sm
     if (!coop)
         return KPP_ERR_UNSUPPORTED;
     const int64_t a = pl->pk.rows_align;
-    const int64_t min_rows = o.min_rows_per_cta > 0 ? o.min_rows_per_cta : 2048;
+    const bool any_d = !pl->pk.fn_smem;
+    // 2048 rows, but no more than 32 KB of them for a wide any-d row (20 000 x
+    // 2000, K = 20 took 4.2 ms on the 10 CTAs of 2048 rows, 2.8 streamed)
+    int64_t few = 2048;
+    if (any_d)
+        while (few > 32 && few * d * elem_bytes(dt) > 32768)
+            few /= 2;
+    const int64_t min_rows = o.min_rows_per_cta > 0 ? o.min_rows_per_cta : few;
     const int64_t target = (int64_t)sms * per_sm;
     int64_t chunk = (N + target - 1) / target;
     if (chunk < min_rows)
@@ -180,7 +187,7 @@ kpp_status plan_persistent_at(int64_t N, int32_t K, const kpp_options &o, int sm
         return KPP_ERR_UNSUPPORTED;
     // shared memory: D^2 of the block if it fits, then as many cached rows as fit
     cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, pl->pk.fn_smem) != cudaSuccess)
+    if (cudaFuncGetAttributes(&fa, any_d ? pl->pk.prune_smem : pl->pk.fn_smem) != cudaSuccess)
         return KPP_ERR_CUDA;
     const int64_t budget = ((int64_t)optin - (int64_t)fa.sharedSizeBytes - 1024) / per_sm;
     int64_t used = 0;
@@ -195,7 +202,7 @@ kpp_status plan_persistent_at(int64_t N, int32_t K, const kpp_options &o, int sm
     const int64_t seg_supers = ((chunk / a) + nseg - 1) / nseg; // longest segment
     const int64_t unit = (int64_t)nseg * a * pl->pk.row_bytes;  // one super per warp
     int64_t supers = 0;
-    if (o.smem_cache >= 0) {
+    if (o.smem_cache >= 0 && !any_d) {
         supers = (budget - used) / unit;
         if (supers > seg_supers)
             supers = seg_supers;
@@ -205,25 +212,39 @@ kpp_status plan_persistent_at(int64_t N, int32_t K, const kpp_options &o, int sm
             supers = 0;
     }
     pl->psmem = (size_t)(supers * unit + (d2_in_smem ? d2_bytes : 0));
-    // Passes that skip rows, unless the caller asked for a point cache or the
-    // whole block fits one (its passes then read no row from L2 at all).
+    // Passes that skip rows, unless the caller asked for a point cache or half
+    // of the block fits one (6 020 x 64 BF16, K = 993: 7.3 ms with 80 % of the
+    // rows cached, 8.7 skipping; 100 000 x 64 FP32, K = 100, 40 %: 968 / 842 us).
     // Below kPruneMinK passes too few come after the first seeds, which can
     // skip little (10^6 x 32, K = 256: 0.99 of the rows are read at pass 1,
     // 0.78 at 25, 0.26 at 128).
     pl->prune = false;
-    if (pl->pk.prune_smem && K >= kPruneMinK && per_sm == 1 && o.smem_cache <= 0 &&
-        supers < seg_supers) {
-        const PruneLayout in = prune_layout(d2_bytes, chunk, K, true, nseg);
-        d2_in_smem = d2_in_smem && in.bytes <= budget;
+    bool skip = K >= kPruneMinK && o.smem_cache <= 0 && 2 * supers < seg_supers;
+    if (pl->pk.prune_smem && per_sm == 1 && (skip || any_d)) {
+        const int64_t cen = any_d ? generic_centre_floats(dt, d) : 0;
+        const PruneLayout in = prune_layout(d2_bytes, chunk, K, true, nseg, cen);
+        const bool in_smem = d2_in_smem && in.bytes <= budget;
+        // D^2 leaving shared memory for the lists costs a short seeding more
+        // than it skips (4 10^6 x 32, K = 8: 609 -> 659 us; K = 30: 1446 -> 1241
+        // at d = 16)
+        if (d2_in_smem && !in_smem && !any_d && K < 2 * kPruneMinK)
+            skip = false;
         const int64_t bytes =
-            d2_in_smem ? in.bytes : prune_layout(0, chunk, K, false, nseg).bytes;
-        pl->prune = bytes <= budget;
-        if (pl->prune) {
+            in_smem ? in.bytes : prune_layout(0, chunk, K, false, nseg, cen).bytes;
+        if (!skip && !any_d) {
+            // the plain kernel
+        } else if (bytes <= budget) {
+            pl->prune = skip;
+            d2_in_smem = in_smem;
             supers = 0;
             pl->psmem = (size_t)bytes;
+        } else if (any_d) {
+            return KPP_ERR_UNSUPPORTED; // the centre's features take the room
         }
+    } else if (any_d) {
+        return KPP_ERR_UNSUPPORTED;
     }
-    if (pl->prune)
+    if (pl->prune || any_d)
         pl->pfn = d2_in_smem ? pl->pk.prune_smem : pl->pk.prune_global;
     else
         pl->pfn = d2_in_smem ? pl->pk.fn_smem : pl->pk.fn_global;
@@ -253,6 +274,20 @@ kpp_status plan_persistent_at(int64_t N, int32_t K, const kpp_options &o, int sm
     return KPP_OK;
 }
 
+// Whether the automatic choice takes the persistent any-d kernel for a d
+// without a specialisation: one launch and rows read in 16-byte chunks in place
+// of K launches that read single elements.  Narrow rows fill few of their
+// chunks, and a short seeding skips few rows.  Streamed / persistent measured
+// (ms): 300 007 x 50 FP32, K = 100 3.19 / 1.62; 60 000 x 784, K = 50 6.9 / 2.5;
+// 5 10^6 x 100, K = 6 4.55 / 2.10; 1.4 10^6 x 20 BF16, K = 21 (40 bytes) 1.09
+// times faster; but 2.7 10^6 x 14 FP32, K = 15 0.79 / 1.09, 1.1 10^6 x 19, K = 9
+// 0.32 / 0.38, 2.8 10^6 x 9 BF16, K = 84 (18 bytes) 2.44 / 2.75.
+bool any_d_rule(int32_t d, int32_t K, int dt)
+{
+    const int rb = d * elem_bytes(dt);
+    return rb >= 40 && (K >= 16 || rb >= 80);
+}
+
 kpp_status make_plan(int64_t N, int32_t d, int32_t K, int dt, const kpp_options *opts, Plan *pl)
 {
     if (!shape_ok(N, d, K, dt))
@@ -261,9 +296,15 @@ kpp_status make_plan(int64_t N, int32_t d, int32_t K, int dt, const kpp_options 
     std::memset(&o, 0, sizeof(o));
     if (opts)
         o = *opts;
+    // The autotuner's choice for this shape.  (It times the forms a caller
+    // can name; for a d without a specialisation that leaves the streamed one,
+    // behind the automatic choice.)
     kpp_options tuned;
-    if (tuned_options(N, d, K, dt, o, &tuned))
-        o = tuned; // the autotuner's choice for this shape
+    PersistentKernel named;
+    if (tuned_options(N, d, K, dt, o, &tuned) &&
+        (tuned.form != KPP_FORM_STREAMED || !any_d_rule(d, K, dt) ||
+         persistent_lookup(dt, d, 0, false, &named)))
+        o = tuned;
     const int sms = device_sms();
     if (sms <= 0)
         return KPP_ERR_CUDA;
@@ -277,14 +318,14 @@ kpp_status make_plan(int64_t N, int32_t d, int32_t K, int dt, const kpp_options 
         return st;
     }
     case KPP_FORM_PERSISTENT:
-        return plan_persistent(N, d, K, dt, o, sms, pl);
+        return plan_persistent(N, d, K, dt, o, sms, false, pl);
     case KPP_FORM_SMALL:
         return plan_small(N, d, dt, pl);
     case KPP_FORM_AUTO: {
         kpp_status st = plan_small(N, d, dt, pl);
         if (st == KPP_OK || st == KPP_ERR_CUDA)
             return st;
-        st = plan_persistent(N, d, K, dt, o, sms, pl);
+        st = plan_persistent(N, d, K, dt, o, sms, any_d_rule(d, K, dt), pl);
         if (st == KPP_OK || st == KPP_ERR_INVALID_ARG || st == KPP_ERR_CUDA)
             return st;
         return plan_streamed(N, d, dt, o, sms, pl);
@@ -520,8 +561,10 @@ kpp_status kpp_seed(const void *points, const float *row_scales, int64_t N, int3
         // no room for the labels (only D^2 in the output array needs it): the
         // kernel that reads every row, with the same blocks
         pl.prune = false;
-        pl.pfn = pl.pk.fn_global;
-        pl.psmem = 0;
+        if (pl.pk.fn_global) {
+            pl.pfn = pl.pk.fn_global;
+            pl.psmem = 0;
+        }
     }
     Problem p;
     std::memset(&p, 0, sizeof(p));

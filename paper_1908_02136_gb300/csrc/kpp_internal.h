@@ -53,7 +53,9 @@ struct PersistentKernel {
     int lanes;
 };
 
-bool persistent_lookup(int dt, int d, int lanes, PersistentKernel *out);
+// any_d: the kernel for every d (no fn_smem / fn_global) where d has no
+// specialisation.
+bool persistent_lookup(int dt, int d, int lanes, bool any_d, PersistentKernel *out);
 int persistent_threads();
 int persistent_max_blocks();
 int persistent_segments();

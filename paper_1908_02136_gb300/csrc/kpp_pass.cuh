@@ -50,6 +50,16 @@ struct Geom {
     static constexpr int PD = WIDE ? PDW : (RPV <= 2 ? 8 : (RPV == 4 ? 4 : 2));
 };
 
+// Any d (D = 0): a lane per row, 32-row groups (GenericPipe below).
+template <int DT> struct Geom<DT, 0, 0> {
+    static constexpr int EB = Fmt<DT>::bytes;
+    static constexpr int EPV = Fmt<DT>::per16;
+    static constexpr int RB = 0;
+    static constexpr bool WIDE = true;
+    static constexpr int L = 0;
+    static constexpr int SW = 32;
+};
+
 // Packed FP32 pairs for the Blackwell FP32x2 instructions.
 using F2 = unsigned long long;
 
@@ -172,6 +182,8 @@ struct PassIO {
     uint16_t *lab;         // nearest centre of every row, indexed by row - r0 (shared
                            //   memory for D2_SMEM, else global), or null
     uint16_t lab_new;      // the label of this pass's centre
+    int d;                 // any-d passes: features, and the bytes of all points
+    int64_t bytes;
 };
 
 __device__ __forceinline__ uint4 ld_global_hint(const void *ptr, uint64_t policy)
@@ -558,9 +570,10 @@ __device__ __forceinline__ Pair pass_rows(const PassIO &io, const CentreRegs<DT,
 // read 34 % of the rows on average (99 % at the first seeds, under 1 % at the
 // last).  Whole seedings before and after: 10^7 x 64, K = 1024 FP32 381 -> 152
 // ms, BF16 225 -> 92 ms; 2 10^7 x 128, K = 2048 FP8 1337 -> 506 ms; 10^6 x 32,
-// K = 256 (in L2) 3.95 -> 3.55 ms; the 512-problem batch 40.6 -> 23.2 ms.  A
-// pass that reads every row costs 394 us here against 370 in the plain kernel
-// (10^7 x 64 FP32), 490 against 652 for FP8 (2 10^7 x 128).
+// K = 256 (in L2) 3.90 -> 3.00 ms; the 512-problem batch 40.6 -> 22.7 ms.
+// Passes that read every row cost what they do in the plain kernel (10^7 x 64,
+// K = 8 without clusters: 3.12 / 3.13 ms; 10^6 x 32: 130 / 140 us), FP8 ones less
+// (2 10^7 x 128: 0.49 / 0.65 ms a pass).
 // ---------------------------------------------------------------------------
 constexpr int kPruneCentres = 2048; // centres with a bound; rows of later ones are always read
 constexpr uint16_t kNoLabel = 0xffff;
@@ -610,13 +623,16 @@ template <int N> __device__ __forceinline__ void cp_async_wait()
 // 8 KB a warp, 128 KB an SM, which is what the plain pass keeps in flight (a
 // register ring beside the list's state spills).  Every lane copies, waits
 // for and reads its own 16-byte vectors, so the ring needs no barrier.  The
-// list grows by whole groups of 32 items; the last one is padded with rows
-// that may be read (n says how many items count).
+// list grows by whole groups of 32 items; n says how many items count, and the
+// last group is read with TAIL, which leaves the items past n out (reading some
+// row in their place put every CTA's padding on the same sectors of L2).
 //   row_at(i, k)     offset in rows from `base` of item i + k (i a multiple of
 //                    32 plus the lane's row group, k a constant below 32)
+//   ahead(own)       called when the group of the lane's own item is issued
+//                    (copies it makes are waited for with the group)
 //   pre(own)         what sink wants of the lane's own item, loaded early
 //   sink(own, v, p)  called on the lane that owns the item
-template <int DT, int D, int L_, class RowAt, class Pre, class Sink> struct RowPipe {
+template <int DT, int D, int L_, class RowAt, class Ahead, class Pre, class Sink> struct RowPipe {
     using G = Geom<DT, D, L_>;
     static_assert(G::WIDE, "rows of at least 16 bytes");
     static constexpr int JB0 = G::VPL >= 4 ? 1 : 4 / G::VPL;
@@ -633,6 +649,7 @@ template <int DT, int D, int L_, class RowAt, class Pre, class Sink> struct RowP
     const float *scales0; // its FP8 scale
     uint32_t ring, sring; // this lane's first vector; the FP8 scales of the rows in flight
     RowAt row_at;
+    Ahead ahead;
     Pre pre;
     Sink sink;
     int n = 0;        // items of the list so far
@@ -642,9 +659,9 @@ template <int DT, int D, int L_, class RowAt, class Pre, class Sink> struct RowP
     float part[G::L]; // this lane's share of each slot's row
 
     __device__ __forceinline__ RowPipe(const PassIO &io, int64_t base,
-                                       const CentreRegs<DT, D, L_> &cr_, char *ring_, RowAt r, Pre p,
-                                       Sink s)
-        : cr(cr_), row_at(r), pre(p), sink(s)
+                                       const CentreRegs<DT, D, L_> &cr_, char *ring_, RowAt r,
+                                       Ahead a, Pre p, Sink s)
+        : cr(cr_), row_at(r), ahead(a), pre(p), sink(s)
     {
         const int lane = threadIdx.x & 31;
         src0 = io.gpts + base * G::RB + (lane % G::L) * 16;
@@ -663,6 +680,7 @@ template <int DT, int D, int L_, class RowAt, class Pre, class Sink> struct RowP
             row[q] = row_at(groups * 32 + g, (jb * JB + q) * (32 / G::L));
     }
 
+    template <bool TAIL>
     __device__ __forceinline__ void issue(int jb, const uint32_t (&row)[JB])
     {
         const uint32_t slot = it & (R - 1);
@@ -670,13 +688,15 @@ template <int DT, int D, int L_, class RowAt, class Pre, class Sink> struct RowP
 #pragma unroll
         for (int q = 0; q < JB; ++q) {
             const char *src = src0 + (uint64_t)row[q] * G::RB;
+            const int i = groups * 32 + (jb * JB + q) * (32 / G::L) + (int)(threadIdx.x & 31) / G::L;
+            if (!TAIL || i < n)
 #pragma unroll
-            for (int v = 0; v < G::VPL; ++v)
-                cp_async16(dst + (q * G::VPL + v) * 512, src + v * G::L * 16);
+                for (int v = 0; v < G::VPL; ++v)
+                    cp_async16(dst + (q * G::VPL + v) * 512, src + v * G::L * 16);
         }
         if constexpr (DT == KPP_FP8_E4M3) {
             const int lane = threadIdx.x & 31;
-            if (BR == 32 || lane < BR)
+            if ((BR == 32 || lane < BR) && (!TAIL || groups * 32 + jb * BR + lane < n))
                 cp_async4(sring + (slot * BR + lane) * 4,
                           scales0 + row_at(groups * 32 + lane, jb * BR));
         }
@@ -740,8 +760,9 @@ template <int DT, int D, int L_, class RowAt, class Pre, class Sink> struct RowP
         }
     }
 
-    // reads the next group of 32 items; the oldest batches in flight make room
-    __device__ __forceinline__ void group()
+    // reads the next group of 32 items (TAIL: those below n); the oldest
+    // batches in flight make room
+    template <bool TAIL> __device__ __forceinline__ void group()
     {
 #pragma unroll
         for (int jb = 0; jb < NB; ++jb) {
@@ -751,7 +772,13 @@ template <int DT, int D, int L_, class RowAt, class Pre, class Sink> struct RowP
                 cp_async_wait<R - 1>();
                 consume((jb + NB * R - R) % NB, R);
             }
-            issue(jb, row);
+            if (jb == 0) {
+                const int lane = threadIdx.x & 31;
+                const int own = groups * 32 + lane % G::L * (32 / G::L) + lane / G::L;
+                if (!TAIL || own < n)
+                    ahead(own);
+            }
+            issue<TAIL>(jb, row);
         }
         ++groups;
     }
@@ -775,12 +802,255 @@ template <int DT, int D, int L_, class RowAt, class Pre, class Sink> struct RowP
     __device__ __forceinline__ bool rest() const { return n > groups * 32; }
 };
 
-template <int DT, int D, int L_, class RowAt, class Pre, class Sink>
-__device__ __forceinline__ RowPipe<DT, D, L_, RowAt, Pre, Sink>
-make_row_pipe(const PassIO &io, int64_t base, const CentreRegs<DT, D, L_> &cr, char *ring, RowAt r,
-              Pre p, Sink s)
+// The row pipe for any d and any row alignment.  A lane owns a row of the
+// 32-row group and adds its features in order -- even ones into one sum, odd
+// ones into the other, as the streamed any-d pass does, bit for bit.  A row's
+// 16-byte chunks (from the 32-byte boundary at or below its first byte) arrive
+// four at a time for all 32 rows: a batch is 2 KB, copied as 64-byte pieces of
+// eight rows per instruction and read back one chunk of one row per lane.  The
+// two halves of a 32-byte sector stay together in shared memory (apart, each
+// is a request of its own to L2); pieces are swizzled by row as far as that
+// allows.  The streamed pass
+// reads single elements a row apart per lane instead: 300 007 x 50, K = 100 32
+// us a pass there, 16 here (bound by shared memory: a batch's chunks are written
+// and read there, and its centre features once per chunk).
+template <int DT, class RowAt, class Ahead, class Pre, class Sink> struct GenericPipe {
+    static constexpr int EB = Fmt<DT>::bytes, EPV = Fmt<DT>::per16;
+    static constexpr int CH = 4;       // chunks per batch
+    static constexpr int BB = 32 * CH * 16;
+    static constexpr int R = kPruneRing / BB; // batches in flight
+    static_assert(R == 4, "four scale slots follow the ring");
+
+    const char *pts;
+    const float *scales;
+    int64_t base;  // first row of the list's base
+    int64_t bytes; // of all points
+    const float *cen; // the centre (FP8: high parts, low parts cen_lo floats on), kCentrePad floats of room before and after
+    int cen_lo;
+    int d, rb, nc, nb; // row bytes; most chunks of a row; batches per group
+    int c_in;          // chunks from here on hold no earlier row's elements
+    uint32_t ring, sring;
+    RowAt row_at;
+    Ahead ahead;
+    Pre pre;
+    Sink sink;
+    int n = 0, groups = 0, done = 0; // items, groups issued and consumed
+    int ib = 0, cb = 0;              // batches of the current group issued and consumed
+    uint32_t it = 0;
+    const char *from[4]; // the rows this lane copies: its chunk of the group's first batch,
+    int left[4], cut[4]; //   chunks from there on, bytes from there to the points' end
+    float a0 = 0.f, a1 = 0.f; // the row being consumed
+    int off = 0;              // elements before its first one in its first chunk
+
+    __device__ __forceinline__ GenericPipe(const PassIO &io, int64_t base_, const float *cen_,
+                                           int cen_lo_, char *ring_, RowAt r, Ahead a, Pre p,
+                                           Sink s)
+        : pts(io.gpts), scales(io.scales), base(base_), bytes(io.bytes), cen(cen_), cen_lo(cen_lo_),
+          d(io.d), rb(io.d * EB), row_at(r), ahead(a), pre(p), sink(s)
+    {
+        // a row starts at a multiple of gcd(rb, 16) past a 32-byte boundary
+        const int g = (rb & -rb) < 16 ? (rb & -rb) : 16;
+        nc = (32 - g + rb + 15) / 16;
+        c_in = g == 16 ? 1 : 2;
+        nb = (nc + CH - 1) / CH;
+        ring = (uint32_t)__cvta_generic_to_shared(ring_);
+        sring = ring + kPruneRing;
+    }
+
+    // bytes between the 32-byte boundary at or below a row's first byte and it
+    __device__ __forceinline__ int lead(int64_t start) const
+    {
+        return (int)((reinterpret_cast<uintptr_t>(pts) + start) & 31);
+    }
+
+    // (a lane's row of the copies and its own row have (lane >> 2) and lane in
+    // place of the swizzle's row; both name the same row's bit)
+    __device__ __forceinline__ static int swizzle(int j, int row) { return j ^ ((row & 2) ? 2 : 0); }
+
+    template <bool TAIL> __device__ __forceinline__ void issue()
+    {
+        const int lane = threadIdx.x & 31, j = lane & 3;
+        const uint32_t dst = ring + (it & (R - 1)) * BB + (lane >> 2) * (CH * 16) +
+                             swizzle(j, lane >> 2) * 16;
+        if (ib == 0) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { // the group's rows this lane copies chunks of
+                const int64_t start = (base + row_at(groups * 32 + (lane >> 2), i * 8)) * rb;
+                const int ld = lead(start);
+                const int64_t at = start - ld + 16 * j;
+                from[i] = pts + at;
+                // chunks from this one to the row's last (none past n); the
+                // last one of all points may be cut short
+                left[i] = TAIL && groups * 32 + (lane >> 2) + i * 8 >= n ? 0 : (ld + rb + 15) / 16 - j;
+                const int64_t rem = bytes - at;
+                cut[i] = (int)(rem < (1 << 20) ? rem : (1 << 20));
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            // (a chunk before the first point: its array need not begin on a
+            // 32-byte boundary)
+            if (left[i] > ib * CH && from[i] + ib * (16 * CH) >= pts) {
+                const int len = cut[i] - ib * (16 * CH);
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                                 dst + i * 8 * (CH * 16)),
+                             "l"(from[i] + ib * (16 * CH)), "r"(len < 16 ? len : 16)
+                             : "memory");
+            }
+        if (ib == 0 && (!TAIL || groups * 32 + lane < n))
+            ahead(groups * 32 + lane);
+        if (DT == KPP_FP8_E4M3 && ib == 0 && (!TAIL || groups * 32 + lane < n))
+            cp_async4(sring + ((groups & 3) * 32 + lane) * 4,
+                      scales + base + row_at(groups * 32 + lane, 0));
+        cp_async_commit();
+        ++it;
+        if (++ib == nb) {
+            ib = 0;
+            ++groups;
+        }
+    }
+
+    // one chunk's elements against the centre's ce[0 ..]; EDGE: only those of
+    // features [0, d) count, e0 being the first element's; PAIR: ce is 8-byte
+    // aligned (d is even)
+    template <bool EDGE, bool PAIR>
+    __device__ __forceinline__ void chunk(const uint4 &x, const float *ce, int e0, float s, F2 &acc) const
+    {
+        float f[EPV];
+        decode16<DT>(x, f);
+#pragma unroll
+        for (int w = 0; w < EPV; w += 2) {
+            float2 h, l;
+            if (PAIR) {
+                h = *reinterpret_cast<const float2 *>(ce + w);
+                if (DT == KPP_FP8_E4M3)
+                    l = *reinterpret_cast<const float2 *>(ce + cen_lo + w);
+            } else {
+                h = make_float2(ce[w], ce[w + 1]);
+                if (DT == KPP_FP8_E4M3)
+                    l = make_float2(ce[cen_lo + w], ce[cen_lo + w + 1]);
+            }
+            F2 t;
+            if constexpr (DT == KPP_FP8_E4M3)
+                t = f2_sub(f2_fma(f2(s, s), f2(f[w], f[w + 1]), f2(-h.x, -h.y)), f2(l.x, l.y));
+            else
+                t = f2_sub(f2(f[w], f[w + 1]), f2(h.x, h.y));
+            if (EDGE) {
+                float t0, t1;
+                f2_split(t, t0, t1);
+                t = f2((unsigned)(e0 + w) < (unsigned)d ? t0 : 0.f,
+                       (unsigned)(e0 + w + 1) < (unsigned)d ? t1 : 0.f);
+            }
+            acc = f2_fma(t, t, acc);
+        }
+    }
+
+    // the first `cnt` of the CH chunks of this lane's row at `src`
+    template <bool EDGE, bool PAIR>
+    __device__ __forceinline__ void chunks(uint32_t src, const float *ceb, int eb, float s, int cnt,
+                                           F2 &acc) const
+    {
+        uint4 x[CH];
+#pragma unroll
+        for (int j = 0; j < CH; ++j)
+            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(x[j].x), "=r"(x[j].y), "=r"(x[j].z), "=r"(x[j].w)
+                         : "r"(src + swizzle(j, threadIdx.x & 31) * 16));
+#pragma unroll
+        for (int j = 0; j < CH; ++j)
+            if (!EDGE || j < cnt)
+                chunk<EDGE, PAIR>(x[j], ceb + j * EPV, eb + j * EPV, s, acc);
+    }
+
+    // the batch issued `back` batches ago
+    __device__ __forceinline__ void consume(uint32_t back)
+    {
+        const int lane = threadIdx.x & 31;
+        __syncwarp(); // other lanes' copies have landed
+        const uint32_t src = ring + ((it - back) & (R - 1)) * BB + lane * (CH * 16);
+        const int own = done * 32 + lane;
+        if (cb == 0) {
+            a0 = a1 = 0.f;
+            off = lead((base + row_at(own, 0)) * rb) / EB;
+        }
+        float s = 1.0f;
+        if constexpr (DT == KPP_FP8_E4M3)
+            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(s) : "r"(sring + ((done & 3) * 32 + lane) * 4));
+        F2 acc = f2(a0, a1);
+        const int eb = cb * CH * EPV - off; // feature of the batch's first element
+        const float *ceb = cen + eb;
+        // one straight run over the batch's chunks either way, so that their
+        // loads overlap
+        const int cnt = nc - cb * CH;
+        if (cb * CH >= c_in && (cb + 1) * CH * 16 <= rb) {
+            if (d & 1)
+                chunks<false, false>(src, ceb, eb, s, cnt, acc);
+            else
+                chunks<false, true>(src, ceb, eb, s, cnt, acc);
+        } else {
+            if (d & 1)
+                chunks<true, false>(src, ceb, eb, s, cnt, acc);
+            else
+                chunks<true, true>(src, ceb, eb, s, cnt, acc);
+        }
+        f2_split(acc, a0, a1);
+        if (++cb == nb) {
+            cb = 0;
+            if (own < n)
+                sink(own, a0 + a1, pre(own));
+            ++done;
+        }
+        __syncwarp(); // read before the slot is filled again
+    }
+
+    template <bool TAIL> __device__ __forceinline__ void group()
+    {
+        for (int b = 0; b < nb; ++b) {
+            if (it >= (uint32_t)R) {
+                cp_async_wait<R - 1>();
+                consume(R);
+            }
+            issue<TAIL>();
+        }
+    }
+
+    __device__ __forceinline__ void drain()
+    {
+        cp_async_wait<0>();
+        for (uint32_t left = it < (uint32_t)R ? it : R; left > 0; --left)
+            consume(left);
+    }
+
+    __device__ __forceinline__ bool full() const { return n - groups * 32 >= 32; }
+    __device__ __forceinline__ bool rest() const { return n > groups * 32; }
+};
+
+// The centre of a pass: registers, or shared memory for any d.
+struct GenericCentre {
+    const float *c; // features from index 0, with kCentrePad floats of room before and after
+    int lo;         // FP8: the low parts start here
+};
+
+template <int DT, int D, int L_, class Centre, class RowAt, class Ahead, class Pre, class Sink>
+__device__ __forceinline__ auto make_row_pipe(const PassIO &io, int64_t base, const Centre &c,
+                                              char *ring, RowAt r, Ahead a, Pre p, Sink s)
 {
-    return RowPipe<DT, D, L_, RowAt, Pre, Sink>(io, base, cr, ring, r, p, s);
+    if constexpr (D == 0)
+        return GenericPipe<DT, RowAt, Ahead, Pre, Sink>(io, base, c.c, c.lo, ring, r, a, p, s);
+    else
+        return RowPipe<DT, D, L_, RowAt, Ahead, Pre, Sink>(io, base, c, ring, r, a, p, s);
+}
+
+// floats before and after a centre in shared memory: a chunk of a row's first
+// or last bytes may reach 31 features before it, one past its last 94 after it
+// (they count nothing)
+constexpr int kCentrePad = 96;
+
+// Shared-memory floats of an any-d centre.
+__host__ __device__ __forceinline__ int64_t generic_centre_floats(int dt, int d)
+{
+    const int64_t one = (d + 2 * kCentrePad + 3) / 4 * 4;
+    return dt == KPP_FP8_E4M3 ? 2 * one : one;
 }
 
 // A row's new D^2 with its previous one given; stores what changed.
@@ -800,11 +1070,11 @@ __device__ __forceinline__ float keep_nearest(const PassIO &io, int64_t row, flo
 
 // Shared memory of the passes that skip rows, beside the block's D^2 and
 // chunk sums (byte offsets from `base`): labels (D^2 in shared memory only),
-// the bounds and rows of the chosen centres, every warp's ring (with room for
-// FP8 scales) and list of rows to read, and (D^2 in the output array only)
+// the bounds and rows of the chosen centres, the pass's centre (any d), every
+// warp's ring (with room for FP8 scales) and list of rows to read, and (D^2 in the output array only)
 // the D^2 of those rows.
 struct PruneLayout {
-    int64_t lab, thr, cidx, ring, list, list_d2, bytes;
+    int64_t lab, thr, cidx, cen, ring, list, list_d2, bytes;
 };
 // (a ring starts on a 128-byte boundary: at 16 bytes past one every 32-byte
 // sector lands in two of shared memory and is requested from L2 twice --
@@ -820,18 +1090,37 @@ template <> struct ListRow<D2_SMEM> {
 };
 
 __host__ __device__ __forceinline__ PruneLayout prune_layout(int64_t base, int64_t chunk, int K,
-                                                             bool d2_in_smem, int nwarps)
+                                                             bool d2_in_smem, int nwarps,
+                                                             int64_t centre_floats = 0)
 {
     PruneLayout p;
     const int64_t kp = K < kPruneCentres ? K : kPruneCentres;
     p.lab = (base + 15) & ~15ll;
     p.thr = p.lab + (d2_in_smem ? ((2 * chunk + 15) & ~15ll) : 0);
     p.cidx = p.thr + 4 * kp;
-    p.ring = (p.cidx + 4 * kp + 127) & ~127ll;
+    p.cen = (p.cidx + 4 * kp + 15) & ~15ll;
+    p.ring = (p.cen + 4 * centre_floats + 127) & ~127ll;
     p.list = p.ring + (int64_t)kPruneRingBytes * nwarps;
     p.list_d2 = p.list + (d2_in_smem ? 2ll : 4ll) * kPruneList * nwarps;
     p.bytes = p.list_d2 + (d2_in_smem ? 0 : 4ll * kPruneList * nwarps);
     return p;
+}
+
+// The end of a pass over a segment: D^2 to the output array where the pass
+// asks for it, the segment's sum.
+template <int MODE>
+__device__ __forceinline__ void pass_end(const PassIO &io, int64_t seg_first, int rows,
+                                         const Pair &lacc)
+{
+    const int lane = threadIdx.x & 31;
+    if (MODE == D2_SMEM && io.d2_out) {
+        __syncwarp(); // the rows' last stores came from other lanes
+        for (int o = lane; o < rows; o += 32)
+            io.d2_out[seg_first + o] = io.d2s[seg_first - io.r0 + o];
+    }
+    const Pair seg = warp_pair_sum(lacc);
+    if (lane == 0)
+        io.segs[threadIdx.x >> 5] = make_float2(seg.hi, seg.lo);
 }
 
 struct PruneIO {
@@ -839,14 +1128,15 @@ struct PruneIO {
     float *thr;          // room for the bounds of the chosen centres (shared memory)
     const int32_t *cidx; // their rows (shared memory)
     int nc;              // chosen centres to take a bound for (0: read every row)
+    float *cen;          // room for the pass's centre (any d; shared)
     char *ring;          // this warp's ring (shared)
     void *list;          // this warp's list of rows to read (shared)
-    float *list_d2;      // their D^2 (D2_INPLACE; shared)
+    float *list_d2;      // their D^2, or that of the rows in flight (D2_INPLACE; shared)
     int *active;         // out: rows each warp read (shared)
 };
 
 // The pass over this warp's segment that reads only the rows whose D^2 can
-// fall (all of them when pr.nc is 0).  A block of 32-row groups at a time:
+// fall, or (pr.nc == 0) all of them.  A block of 32-row groups at a time:
 // their D^2 and labels (the next block's loads are in flight meanwhile) are
 // tested one row per lane, and the rows left go to the warp's list, which
 // feeds the row pipe a full group at a time, so the reads of one block's rows
@@ -865,8 +1155,28 @@ __device__ __forceinline__ void pass_rows_pruned(const PassIO &io, const PruneIO
     segment_rows(io.r0, io.r1 - io.r0, G::SW, nwarps, warp, &seg_first, &seg_last);
     const int rows = (int)(seg_last - seg_first); // offsets in the segment are ints
     const int64_t rel = seg_first - io.r0;
-    CentreRegs<DT, D, L_> cr;
-    cr.load(io.gpts, io.scales, pr.ci);
+    auto centre = [&] {
+        if constexpr (D == 0) {
+            GenericCentre gc;
+            gc.c = pr.cen + kCentrePad;
+            gc.lo = (int)generic_centre_floats(KPP_F32, io.d);
+            const float s = DT == KPP_FP8_E4M3 ? __ldg(io.scales + pr.ci) : 1.0f;
+            for (int k = threadIdx.x; k < io.d; k += blockDim.x) {
+                const float v = decode1<DT>(io.gpts, pr.ci * io.d + k);
+                if constexpr (DT == KPP_FP8_E4M3)
+                    split_fp8_centre(s, v, pr.cen[kCentrePad + k], pr.cen[kCentrePad + gc.lo + k]);
+                else
+                    pr.cen[kCentrePad + k] = v;
+            }
+            __syncthreads();
+            return gc;
+        } else {
+            CentreRegs<DT, D, L_> cr;
+            cr.load(io.gpts, io.scales, pr.ci);
+            return cr;
+        }
+    };
+    const auto cr = centre();
     if (pr.nc > 0) {
         // the distance of the new centre to every chosen one, each warp a
         // share of them
@@ -877,24 +1187,56 @@ __device__ __forceinline__ void pass_rows_pruned(const PassIO &io, const PruneIO
             auto pipe = make_row_pipe<DT, D, L_>(
                 io, 0, cr, pr.ring,
                 [&](int i, int k) { return (uint32_t)pr.cidx[f + (i + k < n ? i + k : n - 1)]; },
-                [](int) { return 0; }, [&](int i, float v, int) { pr.thr[f + i] = prune_bound(v); });
+                [](int) {}, [](int) { return 0; },
+                [&](int i, float v, int) { pr.thr[f + i] = prune_bound(v); });
             pipe.n = n;
             while (pipe.rest())
-                pipe.group();
+                pipe.template group<true>();
             pipe.drain();
         }
         __syncthreads();
     }
+    Pair lacc{};
+    if (pr.nc == 0) {
+        // every row, in order (backwards on reverse passes): no tests, no list;
+        // the previous D^2 comes with the group's rows
+        float *old = pr.list_d2;
+        auto at = [&](int i) { return io.reverse ? rows - 1 - i : i; };
+        auto pipe = make_row_pipe<DT, D, L_>(
+            io, seg_first, cr, pr.ring, [&](int i, int k) { return (uint32_t)at(i + k); },
+            [&](int i) {
+                if (MODE == D2_INPLACE && !io.first)
+                    cp_async4((uint32_t)__cvta_generic_to_shared(old + i % kPruneList),
+                              io.d2 + seg_first + at(i));
+            },
+            [&](int i) {
+                return MODE == D2_INPLACE ? old[i % kPruneList]
+                                          : io.d2s[rel + (i < rows ? at(i) : 0)];
+            },
+            [&](int i, float v, float o) {
+                if (kpp_check(io.ctl, seg_first + at(i) < seg_last, 114))
+                    lacc.add(keep_nearest<MODE>(io, seg_first + at(i), v, o));
+            });
+        pipe.n = rows;
+        while (pipe.full())
+            pipe.template group<false>();
+        if (pipe.rest())
+            pipe.template group<true>();
+        pipe.drain();
+        pass_end<MODE>(io, seg_first, rows, lacc);
+        if (lane == 0)
+            pr.active[warp] = rows;
+        return;
+    }
     Row *list = reinterpret_cast<Row *>(pr.list);
     float *list_d2 = pr.list_d2;
-    Pair lacc{};
     struct Own {
         int row;
         float d2;
     };
     auto pipe = make_row_pipe<DT, D, L_>(
         io, seg_first, cr, pr.ring,
-        [&](int i, int k) { return (uint32_t)list[i % kPruneList + k]; },
+        [&](int i, int k) { return (uint32_t)list[i % kPruneList + k]; }, [](int) {},
         [&](int i) {
             Own o;
             o.row = (int)list[i % kPruneList];
@@ -908,7 +1250,7 @@ __device__ __forceinline__ void pass_rows_pruned(const PassIO &io, const PruneIO
     const int nblock = (rows + 32 * U - 1) / (32 * U);
     float d2[U];
     uint16_t lb[U];
-    auto load = [&](int j) { // (in pass 0 both are still unset, and every row is read)
+    auto load = [&](int j) {
         const int b = (io.reverse ? nblock - 1 - j : j) * 32 * U;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -919,7 +1261,7 @@ __device__ __forceinline__ void pass_rows_pruned(const PassIO &io, const PruneIO
                 lb[u] = in ? io.lab[rel + o] : 0;
             } else {
                 d2[u] = in ? __ldcg(io.d2 + seg_first + o) : 0.f;
-                lb[u] = in && pr.nc > 0 ? __ldcg(io.lab + rel + o) : 0;
+                lb[u] = in ? __ldcg(io.lab + rel + o) : 0;
             }
         }
     };
@@ -932,7 +1274,7 @@ __device__ __forceinline__ void pass_rows_pruned(const PassIO &io, const PruneIO
         for (int u = 0; u < U; ++u) {
             const int o = b + 32 * u + lane;
             const float t = lb[u] < pr.nc ? pr.thr[lb[u]] : -1.f;
-            const bool must = o < rows && (io.first || !(d2[u] <= t));
+            const bool must = o < rows && !(d2[u] <= t);
             const unsigned m = __ballot_sync(0xffffffffu, must);
             if (must) {
                 const int at = (n + __popc(m & ((1u << lane) - 1u))) % kPruneList;
@@ -946,28 +1288,21 @@ __device__ __forceinline__ void pass_rows_pruned(const PassIO &io, const PruneIO
         pipe.n = n;
         if (j + 1 < nblock) {
             load(j + 1);
-        } else { // the last group's other items: rows that may be read
+        } else { // the last group's other items are looked at, not read
             list[(n + lane) % kPruneList] = 0;
             if (MODE == D2_INPLACE)
                 list_d2[(n + lane) % kPruneList] = 0.f;
         }
         __syncwarp(); // the list is read by other lanes
         while (pipe.full())
-            pipe.group();
+            pipe.template group<false>();
     }
     if (pipe.rest())
-        pipe.group();
+        pipe.template group<true>();
     pipe.drain();
-    if (MODE == D2_SMEM && io.d2_out) {
-        __syncwarp(); // the rows' last stores came from other lanes
-        for (int o = lane; o < rows; o += 32)
-            io.d2_out[seg_first + o] = io.d2s[rel + o];
-    }
-    const Pair seg = warp_pair_sum(lacc);
-    if (lane == 0) {
-        io.segs[warp] = make_float2(seg.hi, seg.lo);
+    pass_end<MODE>(io, seg_first, rows, lacc);
+    if (lane == 0)
         pr.active[warp] = pipe.n;
-    }
 }
 
 // The CTA's D^2 sum: warp pairs added in warp order, rounded once to FP64.

@@ -5,7 +5,7 @@
 
 namespace kpp {
 
-bool persistent_lookup(int dt, int d, int lanes, PersistentKernel *out)
+bool persistent_lookup(int dt, int d, int lanes, bool any_d, PersistentKernel *out)
 {
     const PSpec *best = nullptr;
     int nf = 0, nb = 0, n8 = 0;
@@ -23,6 +23,10 @@ bool persistent_lookup(int dt, int d, int lanes, PersistentKernel *out)
         if (!best || (s.lanes <= 8 && s.lanes > best->lanes))
             best = &s;
     }
+    if (!best && any_d && lanes <= 0)
+        for (int i = 0; i < ns[dt]; ++i)
+            if (tabs[dt][i].d == 0)
+                best = &tabs[dt][i];
     if (!best)
         return false;
     out->fn_smem = reinterpret_cast<const void *>(best->fn_smem);

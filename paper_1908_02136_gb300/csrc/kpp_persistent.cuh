@@ -59,9 +59,10 @@ struct BlockShared {
     int few;                   // they were few enough to go on skipping
 };
 
-// Passes test for rows to skip while at most kPruneKeep of the block's rows
-// had to be read; above that they read every row -- no bounds to compute, which
-// cost up to 10 us at 1000 centres -- and every kPruneProbe-th pass tests again.
+// Passes test for rows to skip while the rows read, the chosen centres' (for
+// their bounds) included, were at most kPruneKeep of the block's; above that
+// they read every row, and every kPruneProbe-th pass tests again as long as the
+// bounds are a small part of it.
 constexpr float kPruneKeep = 0.8f;
 constexpr int kPruneProbe = 8;
 
@@ -101,7 +102,8 @@ __device__ __forceinline__ void seed_blocks(const Problem &p, const PersistArgs 
         pl = prune_layout(MODE == D2_SMEM
                               ? ((4 * p.chunk + 15) & ~15ll) + 8 * ((p.chunk + 31) / 32)
                               : 0,
-                          p.chunk, p.K, MODE == D2_SMEM, kPersistWarps);
+                          p.chunk, p.K, MODE == D2_SMEM, kPersistWarps,
+                          D == 0 ? generic_centre_floats(DT, p.d) : 0);
     float *thr = reinterpret_cast<float *>(smem + pl.thr);
     int32_t *cidx = reinterpret_cast<int32_t *>(smem + pl.cidx);
     if (threadIdx.x == 0)
@@ -147,13 +149,15 @@ __device__ __forceinline__ void seed_blocks(const Problem &p, const PersistArgs 
         io.d2s = d2s;
         io.segs = segsum;
         io.policy = policy;
+        io.d = p.d;
+        io.bytes = p.N * p.d * G::EB;
         bool prune = false;
         if constexpr (PRUNE) {
             if (can_prune) {
                 io.lab = MODE == D2_SMEM ? reinterpret_cast<uint16_t *>(smem + pl.lab)
                                          : p.labels + r0;
                 io.lab_new = m < kPruneCentres ? (uint16_t)m : kNoLabel;
-                prune = m > 0 && (sh.few || m % kPruneProbe == 1);
+                prune = m > 0 && (sh.few || (m % kPruneProbe == 1 && 4 * m <= r1 - r0));
                 if (threadIdx.x == 0 && m < kPruneCentres)
                     cidx[m] = (int32_t)ci; // read from the next pass on
             }
@@ -162,6 +166,7 @@ __device__ __forceinline__ void seed_blocks(const Problem &p, const PersistArgs 
             pr.thr = thr;
             pr.cidx = cidx;
             pr.nc = !prune ? 0 : (m < kPruneCentres ? m : kPruneCentres);
+            pr.cen = reinterpret_cast<float *>(smem + pl.cen);
             pr.ring = smem + pl.ring + warp * kPruneRingBytes;
             pr.list = smem + pl.list + warp * kPruneList * (int)sizeof(typename ListRow<MODE>::type);
             pr.list_d2 = reinterpret_cast<float *>(smem + pl.list_d2) + warp * kPruneList;
@@ -238,7 +243,8 @@ __device__ __forceinline__ void seed_blocks(const Problem &p, const PersistArgs 
                 int read = 0;
                 for (int w = 0; w < kPersistWarps; ++w)
                     read += sh.active[w];
-                sh.few = (float)read <= kPruneKeep * (float)(r1 - r0);
+                // (the bounds of the chosen centres are rows read too)
+                sh.few = (float)(read + m) <= kPruneKeep * (float)(r1 - r0);
             }
             if (chunk_path && !forced) {
                 for (int c = threadIdx.x - 32; c < nchunks; c += blockDim.x - 32) {
@@ -424,6 +430,15 @@ constexpr PSpec make_pspec()
         s.prune_global = &persistent_kernel<DT, D, L, D2_INPLACE, true>;
     }
     return s;
+}
+
+// The any-d kernel (always with the passes that skip rows).
+template <int DT>
+constexpr PSpec make_pspec_generic()
+{
+    using G = Geom<DT, 0, 0>;
+    return PSpec{DT, 0, 0, G::SW, 0, nullptr, nullptr, &persistent_kernel<DT, 0, 0, D2_SMEM, true>,
+                 &persistent_kernel<DT, 0, 0, D2_INPLACE, true>};
 }
 
 // The specialisations built for each stored type (one translation unit each,

@@ -15,6 +15,7 @@ const PSpec kSpecs[] = {
     make_pspec<KPP_BF16, 64, 8>(),
     make_pspec<KPP_BF16, 128, 4>(),
     make_pspec<KPP_BF16, 128, 8>(),
+    make_pspec_generic<KPP_BF16>(),
 };
 } // namespace
 

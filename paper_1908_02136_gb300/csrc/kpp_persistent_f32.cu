@@ -16,6 +16,7 @@ const PSpec kSpecs[] = {
     make_pspec<KPP_F32, 64, 8>(),
     make_pspec<KPP_F32, 128, 4>(),
     make_pspec<KPP_F32, 128, 8>(),
+    make_pspec_generic<KPP_F32>(),
 };
 } // namespace
 

@@ -12,6 +12,7 @@ const PSpec kSpecs[] = {
     make_pspec<KPP_FP8_E4M3, 32, 2>(),
     make_pspec<KPP_FP8_E4M3, 64, 4>(),
     make_pspec<KPP_FP8_E4M3, 128, 8>(),
+    make_pspec_generic<KPP_FP8_E4M3>(),
 };
 } // namespace
 

@@ -144,3 +144,38 @@ def test_bound_never_skips_a_nearer_row():
                                  f(-1))
             skipped = d2 <= bound
             assert not (v[skipped] < d2[skipped]).any()
+
+
+# any d (the automatic choice; a named form still refuses or streams it): rows
+# at every alignment, one chunk to many, the last row ending inside a chunk
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", ["f32", "bf16", "fp8"])
+@pytest.mark.parametrize("N,d", [(120_001, 1), (60_001, 3), (40_003, 5), (30_001, 7), (20_011, 12),
+                                 (20_001, 15), (20_003, 17), (9_001, 33), (9_003, 50), (5_001, 100),
+                                 (5_003, 129), (3_001, 300), (2_500, 784), (601, 4095), (700, 4096)])
+def test_any_width_same_as_the_streamed_form(N, d, dtype):
+    x = datagen.gmm(N, d, 12, seed=N + d, outlier_frac=0.05)
+    q, s = _stored(x, dtype)
+    for K in (5, 40):
+        ref = kpp.seed(q, K, 3, dtype=dtype, row_scales=s, opts={"form": kpp.FORM_STREAMED})
+        for opts in (None, {"min_rows_per_cta": 70_000}):  # D^2 in shared memory / in the output
+            _same(ref, kpp.seed(q, K, 3, dtype=dtype, row_scales=s, opts=opts))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("d", [32, 50])
+def test_seeding_inside_a_captured_graph(d):
+    x = torch.from_numpy(datagen.gmm(60_000, d, 16, seed=d)).to(DEV)
+    ref = kpp.seed(x, 24, 3)
+    ws = kpp.workspace_for(60_000, d, 24, kpp.F32, x.device)
+    out = tuple(torch.zeros_like(t) for t in ref)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        kpp.seed(x, 24, 3, workspace=ws, out=out, check=False)
+    for _ in range(2):
+        for t in out:
+            t.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        for a, b in zip(ref, out):
+            assert torch.equal(a, b)
