@@ -129,11 +129,14 @@ kpp_status make_batch_plan(const kpp_problem *pr, int32_t n, int dt, const kpp_o
     const int grid = sms; // one CTA per SM
     const int64_t min_rows = (opts && opts->min_rows_per_cta > 0) ? opts->min_rows_per_cta : 2048;
     const double eb = elem_bytes(dt);
-    // Cost model, in bytes-equivalents: the points read per pass, D^2 read and
-    // written per pass, and a fixed per-pass cost of the exchange.
+    // Cost model, in bytes at an SM's share of HBM: the share of the points a
+    // pass reads once rows are skipped, D^2 and labels tested for every row,
+    // and a fixed cost per pass (bounds, exchange and draw).  The 512-problem
+    // batch takes 22.6 ms with the model of passes that read everything (1, 8
+    // bytes; 64, 256 KB), 22.0 with 200 and 400 KB a pass, 21.4 with these.
     auto cost_of = [&](int i, int t) {
         const double rows = (double)pr[i].N / t;
-        return (double)pr[i].K * (rows * (pr[i].d * eb + 8.0) + (t > 1 ? 256.0e3 : 64.0e3));
+        return (double)pr[i].K * (rows * (0.4 * pr[i].d * eb + 24.0) + (t > 1 ? 600.0e3 : 300.0e3));
     };
     std::vector<double> c1(n);
     for (int i = 0; i < n; ++i)
