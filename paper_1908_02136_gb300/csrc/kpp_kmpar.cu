@@ -498,7 +498,11 @@ __global__ void kmpar_weights_out_kernel(const unsigned long long *w, int64_t n,
 // stop: the remaining indices are -1.
 // ---------------------------------------------------------------------------
 constexpr int kRecMaxCluster = 16;
-constexpr int kRecPerCta = 512; // target candidates per CTA
+// Target candidates per CTA.  Fewer put less on a draw's chain of distances,
+// more CTAs in its two barriers: 2 626 x 32, K = 256 963 us at 176, 871 at 300,
+// 913 at 512, 1 049 at 1 000; 5 001 x 128, K = 500 2.50 ms at 300 (the slices'
+// coordinates fit shared memory), 3.92 at 512.
+constexpr int kRecPerCta = 300;
 
 struct RecArgs {
     const float *cT; // [d][ldc] candidate coordinates, feature-major
