@@ -454,12 +454,41 @@ __global__ void __launch_bounds__(kThreads)
         part[blockIdx.x] = t;
 }
 
-// Step 3: weights = histogram of the nearest-candidate positions.
-__global__ void kmpar_weights_kernel(const int32_t *lab, int64_t N, unsigned long long *w)
+// Step 3: weights = histogram of the nearest-candidate positions, counted in
+// shared memory per CTA while the candidates fit (10^7 points, 10 082
+// candidates: 131 us with an atomic per point in L2, 16 so).  160 KB of counters
+// leave one CTA of 1024 threads per SM; more candidates than those are counted
+// in global memory.
+constexpr size_t kWeightsSmem = 160 * 1024;
+constexpr int kWeightsThreads = 1024;
+
+__global__ void __launch_bounds__(kWeightsThreads)
+    kmpar_weights_kernel(const int32_t *lab, int64_t N, int nc, unsigned long long *w)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N;
-         i += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(&w[lab[i]], 1ull);
+    extern __shared__ unsigned wcnt[]; // [nc], or none: counted in global memory
+    const bool local = (size_t)nc * 4 <= kWeightsSmem;
+    for (int k = threadIdx.x; local && k < nc; k += blockDim.x)
+        wcnt[k] = 0u;
+    __syncthreads();
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i0 < N; i0 += 4 * step) {
+        int32_t l[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            l[u] = i0 + u * step < N ? __ldg(lab + i0 + u * step) : -1;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (l[u] >= 0) {
+                if (local)
+                    atomicAdd(wcnt + l[u], 1u);
+                else
+                    atomicAdd(&w[l[u]], 1ull);
+            }
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; local && k < nc; k += blockDim.x)
+        if (wcnt[k])
+            atomicAdd(&w[k], (unsigned long long)wcnt[k]);
 }
 
 __global__ void kmpar_weights_out_kernel(const unsigned long long *w, int64_t n, int64_t *out)
@@ -957,7 +986,11 @@ kpp_status kpp_kmeans_par(const float *points, int64_t N, int32_t d, int32_t K, 
     *n_cand_out = nc;
     if (cudaMemsetAsync(wts, 0, (size_t)nc * 8, s) != cudaSuccess)
         return KPP_ERR_CUDA;
-    kmpar_weights_kernel<<<kGrid, kThreads, 0, s>>>(lab, N, wts);
+    const size_t wsmem = (size_t)nc * 4 <= kWeightsSmem ? (size_t)nc * 4 : 0;
+    if (cudaFuncSetAttribute(kmpar_weights_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kWeightsSmem) != cudaSuccess)
+        return KPP_ERR_CUDA;
+    kmpar_weights_kernel<<<sm_count(), kWeightsThreads, wsmem, s>>>(lab, N, (int)nc, wts);
     RecShape rs;
     if (!rec_shape(nc, d, rec_max_cluster(), &rs))
         return KPP_ERR_UNSUPPORTED;
