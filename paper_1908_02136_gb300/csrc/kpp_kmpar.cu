@@ -527,11 +527,17 @@ __global__ void kmpar_weights_out_kernel(const unsigned long long *w, int64_t n,
 // stop: the remaining indices are -1.
 // ---------------------------------------------------------------------------
 constexpr int kRecMaxCluster = 16;
-// Target candidates per CTA.  Fewer put less on a draw's chain of distances,
-// more CTAs in its two barriers: 2 626 x 32, K = 256 963 us at 176, 871 at 300,
-// 913 at 512, 1 049 at 1 000; 5 001 x 128, K = 500 2.50 ms at 300 (the slices'
-// coordinates fit shared memory), 3.92 at 512.
+// Candidates per CTA.  Fewer put less on a draw's chain of distances, more CTAs
+// in its two barriers, and clusters of 9, 13 and more CTAs pay a step each: up
+// to 8 CTAs of 300, then slices grow to 384 (the most whose coordinates fit
+// shared memory at 128 features), on to 12 CTAs, then all 16.  Whole calls at
+// 30 000 points, us with 7 / 8 / 9 / 12 / 13 / 16 CTAs:
+//   2 412 x 32, K = 256    1327 / 1311 / 1316 / 1354 / 1416 / 1464
+//   2 417 x 128, K = 256   1756 / 1713 / 1737 / 1742 / 1804 / 1831 (6: 2404, not staged)
+//   4 277 x 4, K = 433     1847 / 1833 / 1797 / 1783 / 1895 / 1883
+//   4 042 x 100, K = 433   3702 / 3646 / 2580 / 2549 / 2581 / 2485
 constexpr int kRecPerCta = 300;
+constexpr int kRecPerCtaMost = 384;
 
 struct RecArgs {
     const float *cT; // [d][ldc] candidate coordinates, feature-major
@@ -773,6 +779,10 @@ bool rec_shape(int64_t nc, int d, int max_cluster, RecShape *out)
 {
     RecShape r;
     r.C = (int)((nc + kRecPerCta - 1) / kRecPerCta);
+    if (r.C > 8) {
+        const int64_t wide = (nc + kRecPerCtaMost - 1) / kRecPerCtaMost;
+        r.C = wide <= 8 ? 8 : (wide <= 12 ? (int)wide : kRecMaxCluster);
+    }
     r.C = r.C < 1 ? 1 : (r.C > max_cluster ? max_cluster : r.C);
     r.S = (nc + r.C - 1) / r.C;
     r.T = (int)((r.S + 31) / 32 * 32);
