@@ -119,6 +119,10 @@ KERNEL_SOURCES = {
 }
 
 
+# dynamic shared memory of the row rings and lists alone (16 warps)
+ROW_LIST_SMEM = 16 * (8192 + 512 + 2 * 512)
+
+
 def kernel_source_hash(kind: str = "persistent"):
     """SHA-256 over one kernel's CUDA sources (to tell whether a committed ncu
     traffic figure still describes the kernel being run)."""
@@ -503,6 +507,7 @@ def run_batch(args, rank, world, dev, pg, barrier):
             "gpu_launches": args.steps * n_waves,
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic,
+                         "skips_rows": True,
                          "kernel": "batched_kernel (all waves of one step)",
                          "algorithmic_bytes_per_launch": alg_bytes,
                          "algorithmic_bytes_all_ranks": alg_bytes_all},
@@ -621,7 +626,7 @@ def run_lloyd(args, rank, world, dev, pg, barrier):
     ms = total_ms / args.steps
     a_ms = statistics.fmean(assign_ms)
     nkd = float(N) * K * d
-    dp = 64 if d <= 64 else 128
+    dp = -(-d // 16) * 16  # features the MMAs are issued for, 16 a step
     kpad = (K + 127) // 128 * 128
     tensor_flops = 3 * 2.0 * N * kpad * dp  # hi.hi + hi.lo + lo.hi, padded tiles
     peaks = measured_peaks()
@@ -654,7 +659,9 @@ def run_lloyd(args, rank, world, dev, pg, barrier):
                        "assign_ms": a_ms, "parallelism": f"replicas{world}",
                        "l2": "flushed between steps (512 MiB write)",
                        "phi": float(phi.item())},
-            "clocks": clocks, "e2e": None, "gpu_launches": 5 * args.steps,
+            "clocks": clocks, "e2e": None,
+            # centres, assignment, update (count, order, walk; or one), means
+            "gpu_launches": (6 if N >= 200000 or N * d >= 10**7 else 4) * args.steps,
             "roofline": {"bound": "tensor", "achieved": achieved, "peak": peak,
                          "unit": "TFLOP/s", "frac": achieved / peak, "traffic": None,
                          "kernel": "lloyd_assign_pair_kernel",
@@ -737,7 +744,7 @@ def run_kmpar(args, rank, world, dev, pg, barrier):
     total_ms = multi.max_over_ranks(sum(step_ms), pg, dev)
     ms = total_ms / args.steps
     nkd = float(N) * K * d
-    dp = 64 if d <= 64 else 128
+    dp = -(-d // 16) * 16  # features the MMAs are issued for, 16 a step
     kpad = (ke + 127) // 128 * 128
     tensor_flops = 3 * 2.0 * N * kpad * dp
     peaks = measured_peaks()
@@ -759,7 +766,7 @@ def run_kmpar(args, rank, world, dev, pg, barrier):
                          f"{len(o['cand'])} candidates, serial FP64",
                "seconds": dt, "host_cores": cores, "cpu": model}
     if rank == 0:
-        launches = 7 + 8 * R  # prepare, c_0, phi; 8 per round; weights, transpose, recluster, out
+        launches = 7 + 7 * R  # prepare, c_0, phi; 7 per round; weights, transpose, recluster, out
         print(json.dumps({
             "metric": "k-means|| initialisation N*K*d/s (oversampling + weighted recluster)",
             "value": nkd * world * args.steps / (total_ms / 1e3), "unit": "N*K*d/s",
@@ -816,6 +823,7 @@ def roofline_for(plan, form_name, N, d, K, eb, has_scales, ms_per_step, wl_name,
     Algorithmic bytes per pass = the points (N*d*b, plus 4N for FP8 scales),
     plus the 8N bytes of D^2 read and written where D^2 lives in global memory
     (streamed form; persistent form without room for D^2 in shared memory).
+    Plans whose passes skip rows read less (`skips_rows`).
     The bound is L2 when that working set fits the L2 (the persistent form
     keeps it there with an evict-last policy), HBM otherwise; `peak` is the
     measured copy bandwidth of MEASURED_PEAKS.json for HBM and the live
@@ -856,6 +864,12 @@ def roofline_for(plan, form_name, N, d, K, eb, has_scales, ms_per_step, wl_name,
         r["l2_read_gbs"] = peaks_live["l2_read_gbs"]
     if traffic is not None:
         r["traffic_over_algorithmic"] = traffic / alg_bytes
+    # persistent plans without a point cache but with the row lists' shared
+    # memory skip the rows a new seed cannot bring nearer (exactly: D^2 and the
+    # draws keep every bit), so these bytes are what passes over all points
+    # would read: `achieved` is an equivalent rate and may exceed the peak
+    r["skips_rows"] = (form_name == "persistent" and plan["cached_rows_per_cta"] == 0 and
+                       plan["smem_bytes"] >= ROW_LIST_SMEM)
     return r
 
 
@@ -1040,7 +1054,7 @@ def run_seeding(args, rank, world, local, dev, pg, barrier):
                                   ("bound", "achieved", "peak", "frac", "traffic",
                                    "traffic_over_algorithmic", "frac_of_hbm_read",
                                    "frac_of_nominal_hbm", "us_per_pass",
-                                   "algorithmic_bytes_per_pass")
+                                   "algorithmic_bytes_per_pass", "skips_rows")
                                   if k in froof}}
             if not args.no_phi:
                 entry["phi"] = phi_gate(fd, fr)
