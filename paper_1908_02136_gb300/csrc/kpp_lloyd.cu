@@ -1233,7 +1233,9 @@ __global__ void __launch_bounds__(kSegThreads, kSegCtas)
             p = e;
 #pragma unroll
             for (int t = 0; t < VEC; ++t) {
-                double v = (double)hi[t] + (double)lo[t];
+                // (a sum that left the FP32 range is infinite or NaN; its low part,
+                // inf - inf, says nothing)
+                double v = (double)hi[t] + (isfinite(hi[t]) ? (double)lo[t] : 0.0);
 #pragma unroll
                 for (int o = LD; o < 32; o <<= 1)
                     v += __shfl_xor_sync(0xffffffffu, v, o);
