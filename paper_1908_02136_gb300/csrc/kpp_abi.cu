@@ -325,7 +325,9 @@ kpp_status make_plan(int64_t N, int32_t d, int32_t K, int dt, const kpp_options 
         kpp_status st = plan_small(N, d, dt, pl);
         if (st == KPP_OK || st == KPP_ERR_CUDA)
             return st;
-        st = plan_persistent(N, d, K, dt, o, sms, any_d_rule(d, K, dt), pl);
+        // (the any-d kernel runs one CTA per SM: a caller who asks for more gets
+        // the streamed form's grid of that size)
+        st = plan_persistent(N, d, K, dt, o, sms, o.ctas_per_sm <= 1 && any_d_rule(d, K, dt), pl);
         if (st == KPP_OK || st == KPP_ERR_INVALID_ARG || st == KPP_ERR_CUDA)
             return st;
         return plan_streamed(N, d, dt, o, sms, pl);
