@@ -156,9 +156,10 @@ KPP_API int32_t kpp_version(void);
 
 /*
  * Bytes of device workspace for kpp_seed and this problem on the current
- * device (0 if the arguments are invalid).  The size depends on N, d, K,
- * dtype, the options and the device's SM count, not on the data.  Where D^2
- * does not fit shared memory it holds a 16-bit label per point, which lets a
+ * device (0 if the arguments are invalid).  The size depends on N, d, dtype,
+ * the options and the device's SM count, not on the data, and a workspace
+ * sized for one K serves every K of that shape.  Where D^2 may not fit shared
+ * memory it holds a 16-bit label per point, which lets a
  * pass skip the rows it cannot change; a workspace of kpp_describe's
  * workspace_bytes leaves them out: the same results, every row read.
  */

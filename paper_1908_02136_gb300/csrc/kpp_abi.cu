@@ -47,9 +47,10 @@ struct Plan {
     bool prune; // persistent form: passes skip the rows they cannot change
     // workspace layout (byte offsets after the control block)
     size_t off_bsum, off_seg, off_slots;
-    size_t min_bytes; // without the labels of `prune` (a workspace that holds no
-                      // more than these gets the seeding that reads every row)
-    size_t ws_bytes;
+    size_t min_bytes;   // without the labels of `prune` (a workspace that holds no
+                        // more than these gets the seeding that reads every row)
+    size_t label_bytes; // the labels this plan keeps there (0 with D^2 in shared memory)
+    size_t ws_bytes;    // the size to report, which serves every K
 };
 
 bool shape_ok(int64_t N, int32_t d, int32_t K, int dt)
@@ -70,6 +71,7 @@ void layout(Plan *pl, bool persistent)
         pl->off_seg = off;
         off += round_up(sizeof(float2) * (size_t)pl->nblocks * pl->nseg, kAlign);
     }
+    pl->label_bytes = 0;
     pl->min_bytes = pl->ws_bytes = off;
 }
 
@@ -134,6 +136,7 @@ kpp_status plan_small(int64_t N, int32_t d, int dt, Plan *pl)
     pl->sw = 1;
     pl->prune = false;
     pl->off_bsum = pl->off_seg = pl->off_slots = sizeof(Control);
+    pl->label_bytes = 0;
     pl->min_bytes = pl->ws_bytes = sizeof(Control);
     return KPP_OK;
 }
@@ -219,9 +222,16 @@ kpp_status plan_persistent_at(int64_t N, int32_t d, int32_t K, int dt, const kpp
     // skip little (10^6 x 32, K = 256: 0.99 of the rows are read at pass 1,
     // 0.78 at 25, 0.26 at 128).
     pl->prune = false;
-    bool skip = K >= kPruneMinK && o.smem_cache <= 0 && 2 * supers < seg_supers;
+    const bool skippable = pl->pk.prune_smem && per_sm == 1 && o.smem_cache <= 0 &&
+                           2 * supers < seg_supers;
+    bool skip = K >= kPruneMinK && skippable;
+    const int64_t cen = any_d ? generic_centre_floats(dt, d) : 0;
+    // some K keeps the labels in the workspace: D^2 beside the room for the
+    // most bounds does not fit shared memory
+    const bool labels = skippable &&
+                        (!d2_in_smem ||
+                         prune_layout(d2_bytes, chunk, kPruneCentres, true, nseg, cen).bytes > budget);
     if (pl->pk.prune_smem && per_sm == 1 && (skip || any_d)) {
-        const int64_t cen = any_d ? generic_centre_floats(dt, d) : 0;
         const PruneLayout in = prune_layout(d2_bytes, chunk, K, true, nseg, cen);
         const bool in_smem = d2_in_smem && in.bytes <= budget;
         // D^2 leaving shared memory for the lists costs a short seeding more
@@ -269,8 +279,11 @@ kpp_status plan_persistent_at(int64_t N, int32_t d, int32_t K, int dt, const kpp
     pl->pargs.l2_hint = o.l2_policy == 0 ? 1 : (o.l2_policy == 2 ? 2 : 0);
     pl->pargs.timeout_ns = 1000ull * (o.timeout_us ? o.timeout_us : 2000000u);
     layout(pl, true);
+    const size_t label_bytes = round_up(sizeof(uint16_t) * (size_t)N, kAlign);
     if (pl->prune && !d2_in_smem)
-        pl->ws_bytes += round_up(sizeof(uint16_t) * (size_t)N, kAlign); // the labels
+        pl->label_bytes = label_bytes;
+    if (labels)
+        pl->ws_bytes += label_bytes;
     return KPP_OK;
 }
 
@@ -499,7 +512,18 @@ size_t kpp_workspace_size(int64_t N, int32_t d, int32_t K, kpp_dtype dtype,
     Plan pl;
     if (make_plan(N, d, K, (int)dtype, opts, &pl) != KPP_OK)
         return 0;
-    return pl.ws_bytes;
+    size_t bytes = pl.ws_bytes;
+    if (pl.form == KPP_FORM_PERSISTENT && !pl.pk.fn_smem) {
+        // any d: another K of this shape may run the streamed form (any_d_rule)
+        kpp_options o;
+        std::memset(&o, 0, sizeof(o));
+        if (opts)
+            o = *opts;
+        if (plan_streamed(N, d, (int)dtype, o, device_sms(), &pl) != KPP_OK)
+            return 0;
+        bytes = bytes > pl.ws_bytes ? bytes : pl.ws_bytes;
+    }
+    return bytes;
 }
 
 kpp_status kpp_describe(int64_t N, int32_t d, int32_t K, kpp_dtype dtype,
@@ -559,7 +583,7 @@ kpp_status kpp_seed(const void *points, const float *row_scales, int64_t N, int3
         return st;
     if (!workspace || !aligned(workspace, kAlign) || workspace_bytes < pl.min_bytes)
         return KPP_ERR_WORKSPACE;
-    if (pl.prune && workspace_bytes < pl.ws_bytes) {
+    if (pl.prune && workspace_bytes < pl.min_bytes + pl.label_bytes) {
         // no room for the labels (only D^2 in the output array needs it): the
         // kernel that reads every row, with the same blocks
         pl.prune = false;

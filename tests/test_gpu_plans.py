@@ -33,3 +33,35 @@ def test_ctas_per_sm_of_an_automatic_any_d_plan(d, K, ctas):
     ref = kpp.seed(x, K, 3, opts={"form": kpp.FORM_STREAMED})
     out = kpp.seed(x, K, 3, opts={"ctas_per_sm": ctas})
     assert torch.equal(ref[0], out[0]) and torch.equal(ref[1], out[1])
+
+
+# row widths on both sides of every rule of the plans, sets that fit shared
+# memory, L2 and neither
+@pytest.mark.parametrize("dtype", [kpp.F32, kpp.BF16, kpp.FP8_E4M3])
+@pytest.mark.parametrize("d", [2, 8, 10, 14, 19, 32, 33, 50, 70, 100, 128, 300, 785, 2000, 4000])
+def test_a_workspace_sized_for_one_K_serves_every_K(d, dtype):
+    for N in (1500, 3000, 20_000, 65_000, 300_007, 2_000_000, 9_000_000):
+        Ks = [k for k in (1, 4, 7, 8, 15, 16, 20, 100, 1000, 2048, 5000) if k <= N]
+        sizes = [kpp.kpp_workspace_size(N, d, K, dtype) for K in Ks]
+        for K in Ks:
+            st, plan = kpp.kpp_describe(N, d, K, dtype)
+            assert st == kpp.OK
+            assert min(sizes) >= plan.workspace_bytes, (N, K)
+
+
+def test_workspace_sized_for_many_seeds_runs_few():
+    N, d = 20_000, 14
+    x = torch.randn(N, d, device=DEV)
+    ws = kpp.workspace_for(N, d, 100, kpp.F32, x.device)
+    ref = kpp.seed(x, 5, 3, opts={"form": kpp.FORM_STREAMED})
+    out = kpp.seed(x, 5, 3, workspace=ws)
+    assert torch.equal(ref[0], out[0]) and torch.equal(ref[1], out[1])
+
+
+def test_workspace_sized_for_few_seeds_lets_many_skip_rows():
+    """The labels of a plan with D^2 in the output array have their room
+    whatever K the workspace was sized for."""
+    N, d = 4_000_000, 32
+    assert (kpp.kpp_workspace_size(N, d, 4, kpp.F32) ==
+            kpp.kpp_workspace_size(N, d, 64, kpp.F32) >=
+            kpp.kpp_describe(N, d, 64, kpp.F32)[1].workspace_bytes + 2 * N)
