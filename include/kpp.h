@@ -168,8 +168,9 @@ KPP_API size_t kpp_workspace_size(int64_t N, int32_t d, int32_t K, kpp_dtype dty
 
 /*
  * Fills `plan` with the form, grid and memory layout kpp_seed would use for
- * these arguments on the current device.  Host-side only; nothing is
- * launched.  Returns KPP_OK or the error kpp_seed would return.
+ * these arguments on the current device, given kpp_workspace_size bytes of
+ * workspace.  Host-side only; nothing is launched.  Returns KPP_OK or the
+ * error kpp_seed would return.
  */
 KPP_API kpp_status kpp_describe(int64_t N, int32_t d, int32_t K, kpp_dtype dtype,
                                 const kpp_options *opts, kpp_plan *plan);

@@ -106,7 +106,7 @@ kpp_status plan_streamed(int64_t N, int32_t d, int dt, const kpp_options &o, int
 }
 
 kpp_status plan_persistent_at(int64_t N, int32_t d, int32_t K, int dt, const kpp_options &o, int sms,
-                              int per_sm, Plan *pl);
+                              int per_sm, bool may_skip, Plan *pl);
 
 // The small form: one CTA, if the points and D^2 fit its shared memory.
 kpp_status plan_small(int64_t N, int32_t d, int dt, Plan *pl)
@@ -142,9 +142,10 @@ kpp_status plan_small(int64_t N, int32_t d, int dt, Plan *pl)
 }
 
 // The persistent plan at the requested CTAs per SM, or fewer if that many
-// cannot be co-resident.  any_d: also for a d without a specialisation.
+// cannot be co-resident.  any_d: also for a d without a specialisation;
+// may_skip: its passes may skip rows (there is room for the labels).
 kpp_status plan_persistent(int64_t N, int32_t d, int32_t K, int dt, const kpp_options &o, int sms,
-                           bool any_d, Plan *pl)
+                           bool any_d, bool may_skip, Plan *pl)
 {
     if (!persistent_lookup(dt, d, o.lanes_per_row, any_d, &pl->pk))
         return KPP_ERR_UNSUPPORTED;
@@ -153,7 +154,7 @@ kpp_status plan_persistent(int64_t N, int32_t d, int32_t K, int dt, const kpp_op
         return KPP_ERR_INVALID_ARG;
     kpp_status st = KPP_ERR_UNSUPPORTED;
     for (; per_sm >= 1; --per_sm) {
-        st = plan_persistent_at(N, d, K, dt, o, sms, per_sm, pl);
+        st = plan_persistent_at(N, d, K, dt, o, sms, per_sm, may_skip, pl);
         if (st != KPP_ERR_UNSUPPORTED)
             return st;
     }
@@ -161,7 +162,7 @@ kpp_status plan_persistent(int64_t N, int32_t d, int32_t K, int dt, const kpp_op
 }
 
 kpp_status plan_persistent_at(int64_t N, int32_t d, int32_t K, int dt, const kpp_options &o, int sms,
-                              int per_sm, Plan *pl)
+                              int per_sm, bool may_skip, Plan *pl)
 {
     int dev = 0, coop = 0, optin = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -224,7 +225,7 @@ kpp_status plan_persistent_at(int64_t N, int32_t d, int32_t K, int dt, const kpp
     pl->prune = false;
     const bool skippable = pl->pk.prune_smem && per_sm == 1 && o.smem_cache <= 0 &&
                            2 * supers < seg_supers;
-    bool skip = K >= kPruneMinK && skippable;
+    bool skip = K >= kPruneMinK && skippable && may_skip;
     const int64_t cen = any_d ? generic_centre_floats(dt, d) : 0;
     // some K keeps the labels in the workspace: D^2 beside the room for the
     // most bounds does not fit shared memory
@@ -301,7 +302,8 @@ bool any_d_rule(int32_t d, int32_t K, int dt)
     return rb >= 40 && (K >= 16 || rb >= 80);
 }
 
-kpp_status make_plan(int64_t N, int32_t d, int32_t K, int dt, const kpp_options *opts, Plan *pl)
+kpp_status make_plan(int64_t N, int32_t d, int32_t K, int dt, const kpp_options *opts, Plan *pl,
+                     bool may_skip = true)
 {
     if (!shape_ok(N, d, K, dt))
         return KPP_ERR_INVALID_ARG;
@@ -331,7 +333,7 @@ kpp_status make_plan(int64_t N, int32_t d, int32_t K, int dt, const kpp_options 
         return st;
     }
     case KPP_FORM_PERSISTENT:
-        return plan_persistent(N, d, K, dt, o, sms, false, pl);
+        return plan_persistent(N, d, K, dt, o, sms, false, may_skip, pl);
     case KPP_FORM_SMALL:
         return plan_small(N, d, dt, pl);
     case KPP_FORM_AUTO: {
@@ -340,7 +342,8 @@ kpp_status make_plan(int64_t N, int32_t d, int32_t K, int dt, const kpp_options 
             return st;
         // (the any-d kernel runs one CTA per SM: a caller who asks for more gets
         // the streamed form's grid of that size)
-        st = plan_persistent(N, d, K, dt, o, sms, o.ctas_per_sm <= 1 && any_d_rule(d, K, dt), pl);
+        st = plan_persistent(N, d, K, dt, o, sms, o.ctas_per_sm <= 1 && any_d_rule(d, K, dt),
+                             may_skip, pl);
         if (st == KPP_OK || st == KPP_ERR_INVALID_ARG || st == KPP_ERR_CUDA)
             return st;
         return plan_streamed(N, d, dt, o, sms, pl);
@@ -584,13 +587,14 @@ kpp_status kpp_seed(const void *points, const float *row_scales, int64_t N, int3
     if (!workspace || !aligned(workspace, kAlign) || workspace_bytes < pl.min_bytes)
         return KPP_ERR_WORKSPACE;
     if (pl.prune && workspace_bytes < pl.min_bytes + pl.label_bytes) {
-        // no room for the labels (only D^2 in the output array needs it): the
-        // kernel that reads every row, with the same blocks
-        pl.prune = false;
-        if (pl.pk.fn_global) {
-            pl.pfn = pl.pk.fn_global;
-            pl.psmem = 0;
-        }
+        // no room for the labels: the plan that reads every row, with D^2 and the
+        // rows that fit in shared memory (4 10^6 x 32, K = 64 4.7 ms; with D^2 in
+        // the output array and no cache 5.3)
+        st = make_plan(N, d, K, dt, opts, &pl, false);
+        if (st != KPP_OK)
+            return st;
+        if (workspace_bytes < pl.min_bytes)
+            return KPP_ERR_WORKSPACE;
     }
     Problem p;
     std::memset(&p, 0, sizeof(p));
