@@ -123,8 +123,8 @@ kpp_status plan_small(int64_t N, int32_t d, int dt, Plan *pl)
     const size_t smem = small_smem(N, d, dt);
     if (smem + fa.sharedSizeBytes > (size_t)optin)
         return KPP_ERR_UNSUPPORTED; // does not fit one SM
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             optin - (int)fa.sharedSizeBytes) != cudaSuccess)
         return KPP_ERR_CUDA;
     pl->form = KPP_FORM_SMALL;
     pl->pfn = fn;
@@ -259,9 +259,11 @@ kpp_status plan_persistent_at(int64_t N, int32_t d, int32_t K, int dt, const kpp
         pl->pfn = d2_in_smem ? pl->pk.prune_smem : pl->pk.prune_global;
     else
         pl->pfn = d2_in_smem ? pl->pk.fn_smem : pl->pk.fn_global;
-    // static + dynamic shared memory above 48 KB needs the opt-in attribute
+    // static + dynamic shared memory above 48 KB needs the opt-in attribute.  It
+    // belongs to the kernel, not to the call: always the same value, or another
+    // thread's smaller plan would have this one's launch refused.
     if (cudaFuncSetAttribute(pl->pfn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)pl->psmem) != cudaSuccess)
+                             optin - (int)fa.sharedSizeBytes) != cudaSuccess)
         return KPP_ERR_CUDA;
     int resident = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, pl->pfn, persistent_threads(),

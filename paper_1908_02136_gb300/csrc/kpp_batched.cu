@@ -172,8 +172,11 @@ kpp_status make_batch_plan(const kpp_problem *pr, int32_t n, int dt, const kpp_o
                     w.smem, (size_t)prune_layout(0, 0, pr[i].K, false, kPersistWarps).bytes);
         int resident = 0;
         if (!w.fn ||
-            cudaFuncSetAttribute((const void *)w.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)w.smem) != cudaSuccess ||
+            // (the same for every plan: the limit belongs to the kernel, and another
+            // thread's batch of fewer centres must not have this one refused)
+            cudaFuncSetAttribute(
+                (const void *)w.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                (int)prune_layout(0, 0, kPruneCentres, false, kPersistWarps).bytes) != cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, (const void *)w.fn,
                                                           kPersistThreads, w.smem) != cudaSuccess)
             return KPP_ERR_CUDA;

@@ -538,6 +538,7 @@ constexpr int kRecMaxCluster = 16;
 //   4 042 x 100, K = 433   3702 / 3646 / 2580 / 2549 / 2581 / 2485
 constexpr int kRecPerCta = 300;
 constexpr int kRecPerCtaMost = 384;
+constexpr size_t kRecSmem = 200 * 1024; // most dynamic shared memory of a CTA
 
 struct RecArgs {
     const float *cT; // [d][ldc] candidate coordinates, feature-major
@@ -788,10 +789,10 @@ bool rec_shape(int64_t nc, int d, int max_cluster, RecShape *out)
     r.T = (int)((r.S + 31) / 32 * 32);
     r.T = r.T > kRecThreads ? kRecThreads : r.T;
     r.R = (r.S + r.T - 1) / r.T;
-    r.staged = (size_t)r.S * (12 + 4 * (size_t)d) <= 200 * 1024;
+    r.staged = (size_t)r.S * (12 + 4 * (size_t)d) <= kRecSmem;
     r.smem = (size_t)r.S * (r.staged ? 12 + 4 * (size_t)d : 12);
     *out = r;
-    return r.smem <= 200 * 1024;
+    return r.smem <= kRecSmem;
 }
 
 // Largest cluster (16 if the device schedules it, else 8) for this kernel.
@@ -804,7 +805,7 @@ int rec_max_cluster()
     if (cudaFuncSetAttribute(kmpar_recluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed,
                              1) == cudaSuccess &&
         cudaFuncSetAttribute(kmpar_recluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             200 * 1024) == cudaSuccess) {
+                             (int)kRecSmem) == cudaSuccess) {
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -813,7 +814,7 @@ int rec_max_cluster()
         attr[0].val.clusterDim.z = 1;
         cfg.gridDim = dim3(kRecMaxCluster);
         cfg.blockDim = dim3(kRecThreads);
-        cfg.dynamicSmemBytes = 200 * 1024;
+        cfg.dynamicSmemBytes = kRecSmem;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int n = 0;
@@ -828,8 +829,10 @@ int rec_max_cluster()
 
 cudaError_t rec_launch(const RecShape &r, const RecArgs &a, cudaStream_t s)
 {
+    // (the most, whatever this call needs: other threads' calls share the limit)
     cudaError_t e = cudaFuncSetAttribute(kmpar_recluster_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)r.smem);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kRecSmem);
     if (e != cudaSuccess)
         return e;
     if (r.C > 8 && (e = cudaFuncSetAttribute(kmpar_recluster_kernel,

@@ -1355,12 +1355,16 @@ bool make_map(CUtensorMap *m, const void *base, int64_t rows, int dp, int box_ro
                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Most dynamic shared memory of an assignment CTA: the tiles and the norms,
+// 8 KB left free.
+constexpr long long kAssignSmem = 227LL * 1024 - 8 * 1024;
+
 // centre-tile stages that fit beside the point tiles and the centre norms
 int padded_k(int K) { return (K + kBN - 1) / kBN * kBN; }
 
 int assign_stages(int nk, int K, int abufs)
 {
-    const long long budget = 227LL * 1024 - 1024 - 8 * 1024 -
+    const long long budget = kAssignSmem - 1024 -
                              (long long)abufs * kMT * 2 * nk * kABytes - (long long)padded_k(K) * 4;
     const int s = budget > 0 ? (int)(budget / (2 * kBBytes)) : 0;
     return s < kMaxStages ? s : kMaxStages;
@@ -1375,7 +1379,7 @@ int assign_abufs(int nk, int K) { return assign_stages(nk, K, 2) >= kMinStagesTw
 int padded_k_pair(int K) { return (K + kPN - 1) / kPN * kPN; }
 int assign_stages_pair(int nk, int K, int abufs)
 {
-    const long long budget = 227LL * 1024 - 1024 - 8 * 1024 -
+    const long long budget = kAssignSmem - 1024 -
                              (long long)abufs * 2 * nk * kABytes - (long long)padded_k_pair(K) * 4;
     const int s = budget > 0 ? (int)(budget / (2 * kBBytes)) : 0;
     return s < kMaxStagesPair ? s : kMaxStagesPair;
@@ -1446,8 +1450,10 @@ kpp_status assign_impl(const float *centres, const long long *row0, const int32_
         return KPP_ERR_CUDA;
     const int nk = L.dp / kBK;
     const size_t smem = assign_smem(nk, K);
+    // (limits that hold every call: they belong to the kernel, which other threads
+    // launch with other sizes)
     if (cudaFuncSetAttribute(lloyd_assign_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem) != cudaSuccess)
+                             (int)kAssignSmem) != cudaSuccess)
         return KPP_ERR_CUDA;
     AssignArgs a;
     a.N = N;
@@ -1488,7 +1494,7 @@ kpp_status assign_impl(const float *centres, const long long *row0, const int32_
         if (a2.stages >= 2 &&
             cudaFuncSetAttribute(lloyd_assign_pair_kernel,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem2) == cudaSuccess) {
+                                 (int)kAssignSmem) == cudaSuccess) {
             cudaLaunchAttribute attr[1];
             attr[0].id = cudaLaunchAttributeClusterDimension;
             attr[0].val.clusterDim.x = 2;
@@ -1606,7 +1612,7 @@ kpp_status kpp_lloyd_step(const float *points, int64_t N, int32_t d, const float
     const size_t usmem = (size_t)update_tile(K, d) * ((size_t)d * 4 + 4);
     const UpdateFn ufn = update_fn(d);
     if (!ordered && cudaFuncSetAttribute(ufn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)usmem) != cudaSuccess)
+                                         (int)kUpdSmem) != cudaSuccess)
         return KPP_ERR_CUDA;
     auto *ticket = reinterpret_cast<unsigned *>(ws + L.off_ticket);
     if (ordered && cudaMemsetAsync(ticket, 0, sizeof(unsigned), s) != cudaSuccess)
