@@ -112,11 +112,16 @@ typedef struct {
     int32_t use_graph;        /* streamed form: 0/1 = CUDA graph, -1 = plain launches */
     uint32_t timeout_us;      /* persistent form: bound of each grid-barrier wait;
                                  0 = 2,000,000 us */
-    int32_t smem_cache;       /* persistent form: -1 = no shared-memory point cache,
-                                 0 = every row if they all fit (else passes that skip
-                                 rows, or as many rows as fit where those do not
-                                 apply: K < 8, rows under 16 bytes, more than one CTA
-                                 per SM), > 0 = at most this many rows per CTA */
+    int32_t smem_cache;       /* persistent form, the shared-memory point cache and
+                                 which rows a pass reads:
+                                 0 = passes that skip rows, without a cache, unless half
+                                 of the rows or more fit one; where they do not apply
+                                 (K < 8, rows under 16 bytes, more than one CTA per SM)
+                                 a cache of as many rows as fit;
+                                 -1 = no cache (passes skip rows where that applies);
+                                 -2 = no cache, and every pass reads every row;
+                                 > 0 = a cache of at most this many rows per CTA, and
+                                 every pass reads every row */
     int32_t alternate;        /* persistent form: 0/1 = walk rows backwards on odd
                                  passes (L2 reuse), -1 = always forwards */
     int32_t l2_policy;        /* persistent form, streamed rows of plans that read every

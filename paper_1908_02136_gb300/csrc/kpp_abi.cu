@@ -223,8 +223,8 @@ kpp_status plan_persistent_at(int64_t N, int32_t d, int32_t K, int dt, const kpp
     // skip little (10^6 x 32, K = 256: 0.99 of the rows are read at pass 1,
     // 0.78 at 25, 0.26 at 128).
     pl->prune = false;
-    const bool skippable = pl->pk.prune_smem && per_sm == 1 && o.smem_cache <= 0 &&
-                           2 * supers < seg_supers;
+    const bool skippable = pl->pk.prune_smem && per_sm == 1 &&
+                           (o.smem_cache == 0 || o.smem_cache == -1) && 2 * supers < seg_supers;
     bool skip = K >= kPruneMinK && skippable && may_skip;
     const int64_t cen = any_d ? generic_centre_floats(dt, d) : 0;
     // some K keeps the labels in the workspace: D^2 beside the room for the

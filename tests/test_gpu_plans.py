@@ -65,3 +65,31 @@ def test_workspace_sized_for_few_seeds_lets_many_skip_rows():
     assert (kpp.kpp_workspace_size(N, d, 4, kpp.F32) ==
             kpp.kpp_workspace_size(N, d, 64, kpp.F32) >=
             kpp.kpp_describe(N, d, 64, kpp.F32)[1].workspace_bytes + 2 * N)
+
+
+# every pass reading every row, without a cache and with one: the plain plans of
+# a shape whose automatic plan skips rows
+@pytest.mark.parametrize("N,d,dtype", [(300_000, 64, "f32"), (4_000_000, 16, "f32"),
+                                       (300_000, 128, "bf16"), (4_000_000, 16, "fp8")])
+def test_plans_that_read_every_row_can_be_asked_for(N, d, dtype):
+    K = 24
+    code = {"f32": kpp.F32, "bf16": kpp.BF16, "fp8": kpp.FP8_E4M3}[dtype]
+    lists = 16 * 9216  # at least: the row rings and lists of the passes that skip rows
+    st, auto = kpp.kpp_describe(N, d, K, code)
+    assert st == kpp.OK and auto.smem_bytes > lists and auto.cached_rows_per_cta == 0
+    x, scales = torch.randn(N, d, device=DEV), None
+    if dtype == "bf16":
+        x = kpp.quantize(x, dtype)
+    elif dtype == "fp8":
+        x, scales = kpp.quantize(x, dtype)
+    ref = kpp.seed(x, K, 3, row_scales=scales, opts={"form": kpp.FORM_STREAMED})
+    for cache in (-2, 1 << 30):
+        opts = {"form": kpp.FORM_PERSISTENT, "smem_cache": cache}
+        st, plan = kpp.kpp_describe(N, d, K, code, opts)
+        assert st == kpp.OK
+        assert kpp.kpp_workspace_size(N, d, K, code, opts) == plan.workspace_bytes  # no labels
+        assert (plan.cached_rows_per_cta > 0) == (cache > 0)
+        # D^2 stays in shared memory (4 bytes a row and the chunk sums), or all is empty
+        assert plan.d2_in_smem == (plan.rows_per_cta * 4.25 < 220 * 1024)
+        out = kpp.seed(x, K, 3, row_scales=scales, opts=opts)
+        assert torch.equal(ref[0], out[0]) and torch.equal(ref[1], out[1])
