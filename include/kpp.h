@@ -306,17 +306,21 @@ KPP_API kpp_status kpp_seed_batched(const kpp_problem *problems, int32_t n, kpp_
  * points a warp covers per iteration), the smallest row block per CTA, the
  * CTAs per SM of the streamed grid, the persistent form's shared-memory
  * point cache, its L2 policy and traversal, by timing the candidates on the
- * caller's own data: each candidate runs min(K, passes) passes (passes = 0:
- * min(K, 32)) once untimed and twice timed with CUDA events on `stream`;
- * candidates are tried defaults first, and a later one replaces the best so
- * far only if it is more than 1 % faster.
+ * caller's own data: each candidate runs the first min(K, passes) passes
+ * (passes = 0: min(K, 32)) of the seeding of K once untimed and twice timed with
+ * CUDA events on `stream`; candidates are tried defaults first, and a later one
+ * replaces the best so far only if it is more than 1 % faster.  The best plan
+ * whose passes skip rows and the best that reads every row are then compared
+ * over one whole seeding each, since what is skipped depends on the data and
+ * grows with the seeds.
  *   points, row_scales, N, d, K, dtype   as for kpp_seed
  *   indices_out [K], d2_out [N]          device scratch for the trial runs
  *                                        (their contents are undefined after)
  *   workspace   >= kpp_tune_workspace_size(N, d, K, dtype) bytes covers every
  *               candidate; a smaller one skips the candidates it cannot hold
  *   best_out    host: the winning options (form never KPP_FORM_AUTO)
- *   best_ms_per_pass  host, may be NULL: the winner's mean time per pass
+ *   best_ms_per_pass  host, may be NULL: the winner's mean time per pass of
+ *               the first min(K, passes)
  * Blocks the calling thread (it synchronises `stream`).  The winner is also
  * recorded per (device, dtype, d, N, K) for the rest of the process: a later
  * kpp_seed / kpp_workspace_size / kpp_describe for that shape whose options

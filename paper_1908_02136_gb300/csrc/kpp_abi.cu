@@ -468,12 +468,119 @@ kpp_status run_streamed(const Plan &pl, const Problem &p, cudaStream_t stream, i
 
 bool aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
+// What a plan looks like from outside.
+void fill_plan(const Plan &pl, int64_t N, int32_t d, int32_t K, kpp_plan *plan)
+{
+    std::memset(plan, 0, sizeof(*plan));
+    plan->form = pl.form;
+    plan->grid = pl.grid;
+    plan->rows_per_cta = pl.chunk;
+    plan->rows_per_segment = (pl.chunk + pl.nseg - 1) / pl.nseg;
+    plan->workspace_bytes = (int64_t)pl.min_bytes;
+    if (pl.form == KPP_FORM_SMALL) {
+        plan->threads = small_threads();
+        plan->launches = 1;
+        plan->d2_in_smem = 1;
+        plan->cached_rows_per_cta = N;
+        plan->smem_bytes = (int64_t)pl.psmem;
+    } else if (pl.form == KPP_FORM_PERSISTENT) {
+        plan->threads = persistent_threads();
+        plan->launches = 1;
+        plan->lanes_per_row = pl.pk.lanes;
+        plan->d2_in_smem = pl.pfn == pl.pk.fn_smem || pl.pfn == pl.pk.prune_smem ? 1 : 0;
+        plan->cached_rows_per_cta = pl.pargs.cache_supers * pl.nseg * pl.sw;
+        plan->smem_bytes = (int64_t)pl.psmem;
+    } else {
+        plan->threads = streamed_threads();
+        plan->launches = K;
+        plan->lanes_per_row = pl.sk.lanes;
+        plan->smem_bytes = (int64_t)streamed_smem(pl.sk, d);
+    }
+}
+
 } // namespace
 
-bool plan_skips_rows(int64_t N, int32_t d, int32_t K, kpp_dtype dtype, const kpp_options *opts)
+kpp_status plan_facts(int64_t N, int32_t d, int32_t K, kpp_dtype dtype, const kpp_options *opts,
+                      PlanFacts *out)
 {
     Plan pl;
-    return make_plan(N, d, K, (int)dtype, opts, &pl) == KPP_OK && pl.prune;
+    std::memset(&pl, 0, sizeof(pl));
+    const kpp_status st = make_plan(N, d, K, (int)dtype, opts, &pl);
+    if (st != KPP_OK)
+        return st;
+    fill_plan(pl, N, d, K, &out->plan);
+    out->skips = pl.prune;
+    out->bytes = pl.min_bytes + pl.label_bytes;
+    return KPP_OK;
+}
+
+kpp_status seed_passes(const void *points, const float *row_scales, int64_t N, int32_t d,
+                       int32_t K, int32_t passes, kpp_dtype dtype, uint64_t seed,
+                       uint64_t stream_id, const int64_t *forced_prefix, int32_t n_forced,
+                       int64_t *indices_out, float *d2_out, double *phi_out, void *workspace,
+                       size_t workspace_bytes, kpp_stream_t stream, const kpp_options *opts)
+{
+    const int dt = (int)dtype;
+    if (!points || !aligned(points, 16) || !indices_out || !d2_out || !shape_ok(N, d, K, dt))
+        return KPP_ERR_INVALID_ARG;
+    if ((dt == KPP_FP8_E4M3) != (row_scales != nullptr))
+        return KPP_ERR_INVALID_ARG;
+    if (n_forced < 0 || n_forced > K || (n_forced > 0 && !forced_prefix))
+        return KPP_ERR_INVALID_ARG;
+    Plan pl;
+    kpp_status st = make_plan(N, d, K, dt, opts, &pl);
+    if (st != KPP_OK)
+        return st;
+    if (!workspace || !aligned(workspace, kAlign) || workspace_bytes < pl.min_bytes)
+        return KPP_ERR_WORKSPACE;
+    if (pl.prune && workspace_bytes < pl.min_bytes + pl.label_bytes) {
+        // no room for the labels: the plan that reads every row, with D^2 and the
+        // rows that fit in shared memory (4 10^6 x 32, K = 64 4.7 ms; with D^2 in
+        // the output array and no cache 5.3)
+        st = make_plan(N, d, K, dt, opts, &pl, false);
+        if (st != KPP_OK)
+            return st;
+        if (workspace_bytes < pl.min_bytes)
+            return KPP_ERR_WORKSPACE;
+    }
+    Problem p;
+    std::memset(&p, 0, sizeof(p));
+    p.points = points;
+    p.scales = row_scales;
+    p.N = N;
+    p.d = d;
+    p.K = passes; // (shared memory laid out for fewer seeds is within the plan's)
+    p.seed = seed;
+    p.stream_id = stream_id;
+    p.forced = forced_prefix;
+    p.n_forced = n_forced;
+    p.nblocks = pl.nblocks;
+    p.chunk = pl.chunk;
+    p.idx = indices_out;
+    p.d2 = d2_out;
+    p.phi = phi_out;
+    p.nseg = pl.nseg;
+    p.sw = pl.sw;
+    char *ws = reinterpret_cast<char *>(workspace);
+    p.ctl = reinterpret_cast<Control *>(ws);
+    if (pl.form == KPP_FORM_PERSISTENT) {
+        p.slots = reinterpret_cast<unsigned long long *>(ws + pl.off_slots);
+        p.mail = &p.ctl->mail;
+        p.prune = pl.prune ? 1 : 0;
+        p.labels = reinterpret_cast<uint16_t *>(ws + pl.min_bytes);
+    } else {
+        p.block_sums = reinterpret_cast<float2 *>(ws + pl.off_bsum);
+        p.seg_sums = reinterpret_cast<float2 *>(ws + pl.off_seg);
+    }
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    p.recompute = pl.form == KPP_FORM_RECOMPUTE ? 1 : 0;
+    p.exact_draws = (opts && opts->exact_draws) ? 1 : 0;
+    if (pl.form == KPP_FORM_PERSISTENT)
+        return run_persistent(pl, p, s);
+    if (pl.form == KPP_FORM_SMALL)
+        return run_small(pl, p, s);
+    const int use_graph = opts ? opts->use_graph : 0;
+    return run_streamed(pl, p, s, use_graph);
 }
 
 } // namespace kpp
@@ -541,31 +648,7 @@ kpp_status kpp_describe(int64_t N, int32_t d, int32_t K, kpp_dtype dtype,
     kpp_status st = make_plan(N, d, K, (int)dtype, opts, &pl);
     if (st != KPP_OK)
         return st;
-    std::memset(plan, 0, sizeof(*plan));
-    plan->form = pl.form;
-    plan->grid = pl.grid;
-    plan->rows_per_cta = pl.chunk;
-    plan->rows_per_segment = (pl.chunk + pl.nseg - 1) / pl.nseg;
-    plan->workspace_bytes = (int64_t)pl.min_bytes;
-    if (pl.form == KPP_FORM_SMALL) {
-        plan->threads = small_threads();
-        plan->launches = 1;
-        plan->d2_in_smem = 1;
-        plan->cached_rows_per_cta = N;
-        plan->smem_bytes = (int64_t)pl.psmem;
-    } else if (pl.form == KPP_FORM_PERSISTENT) {
-        plan->threads = persistent_threads();
-        plan->launches = 1;
-        plan->lanes_per_row = pl.pk.lanes;
-        plan->d2_in_smem = pl.pfn == pl.pk.fn_smem || pl.pfn == pl.pk.prune_smem ? 1 : 0;
-        plan->cached_rows_per_cta = pl.pargs.cache_supers * pl.nseg * pl.sw;
-        plan->smem_bytes = (int64_t)pl.psmem;
-    } else {
-        plan->threads = streamed_threads();
-        plan->launches = K;
-        plan->lanes_per_row = pl.sk.lanes;
-        plan->smem_bytes = (int64_t)streamed_smem(pl.sk, d);
-    }
+    fill_plan(pl, N, d, K, plan);
     return KPP_OK;
 }
 
@@ -575,67 +658,9 @@ kpp_status kpp_seed(const void *points, const float *row_scales, int64_t N, int3
                     float *d2_out, double *phi_out, void *workspace, size_t workspace_bytes,
                     kpp_stream_t stream, const kpp_options *opts)
 {
-    const int dt = (int)dtype;
-    if (!points || !aligned(points, 16) || !indices_out || !d2_out || !shape_ok(N, d, K, dt))
-        return KPP_ERR_INVALID_ARG;
-    if ((dt == KPP_FP8_E4M3) != (row_scales != nullptr))
-        return KPP_ERR_INVALID_ARG;
-    if (n_forced < 0 || n_forced > K || (n_forced > 0 && !forced_prefix))
-        return KPP_ERR_INVALID_ARG;
-    Plan pl;
-    kpp_status st = make_plan(N, d, K, dt, opts, &pl);
-    if (st != KPP_OK)
-        return st;
-    if (!workspace || !aligned(workspace, kAlign) || workspace_bytes < pl.min_bytes)
-        return KPP_ERR_WORKSPACE;
-    if (pl.prune && workspace_bytes < pl.min_bytes + pl.label_bytes) {
-        // no room for the labels: the plan that reads every row, with D^2 and the
-        // rows that fit in shared memory (4 10^6 x 32, K = 64 4.7 ms; with D^2 in
-        // the output array and no cache 5.3)
-        st = make_plan(N, d, K, dt, opts, &pl, false);
-        if (st != KPP_OK)
-            return st;
-        if (workspace_bytes < pl.min_bytes)
-            return KPP_ERR_WORKSPACE;
-    }
-    Problem p;
-    std::memset(&p, 0, sizeof(p));
-    p.points = points;
-    p.scales = row_scales;
-    p.N = N;
-    p.d = d;
-    p.K = K;
-    p.seed = seed;
-    p.stream_id = stream_id;
-    p.forced = forced_prefix;
-    p.n_forced = n_forced;
-    p.nblocks = pl.nblocks;
-    p.chunk = pl.chunk;
-    p.idx = indices_out;
-    p.d2 = d2_out;
-    p.phi = phi_out;
-    p.nseg = pl.nseg;
-    p.sw = pl.sw;
-    char *ws = reinterpret_cast<char *>(workspace);
-    p.ctl = reinterpret_cast<Control *>(ws);
-    if (pl.form == KPP_FORM_PERSISTENT) {
-        p.slots = reinterpret_cast<unsigned long long *>(ws + pl.off_slots);
-        p.mail = &p.ctl->mail;
-        p.prune = pl.prune ? 1 : 0;
-        p.labels = reinterpret_cast<uint16_t *>(ws + pl.min_bytes);
-    } else {
-        p.block_sums = reinterpret_cast<float2 *>(ws + pl.off_bsum);
-        p.seg_sums = reinterpret_cast<float2 *>(ws + pl.off_seg);
-    }
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    p.recompute = pl.form == KPP_FORM_RECOMPUTE ? 1 : 0;
-    p.exact_draws = (opts && opts->exact_draws) ? 1 : 0;
-    if (pl.form == KPP_FORM_PERSISTENT)
-        return run_persistent(pl, p, s);
-    if (pl.form == KPP_FORM_SMALL)
-        return run_small(pl, p, s);
-    const int use_graph = opts ? opts->use_graph : 0;
-    return run_streamed(pl, p, s, use_graph);
+    return seed_passes(points, row_scales, N, d, K, K, dtype, seed, stream_id, forced_prefix,
+                       n_forced, indices_out, d2_out, phi_out, workspace, workspace_bytes, stream,
+                       opts);
 }
 
 // ---------------------------------------------------------------------------

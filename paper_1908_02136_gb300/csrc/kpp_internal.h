@@ -67,9 +67,20 @@ cudaError_t persistent_launch(const void *fn, int grid, size_t smem, const Probl
 bool tuned_options(int64_t N, int32_t d, int32_t K, int dt, const kpp_options &asked,
                    kpp_options *out);
 
-// Whether kpp_seed's passes skip rows (kpp_pass.cuh) under this plan, given
-// kpp_workspace_size bytes of workspace.
-bool plan_skips_rows(int64_t N, int32_t d, int32_t K, kpp_dtype dtype, const kpp_options *opts);
+// For the autotuner: what kpp_seed does under these options, given the room,
+// and the first `passes` passes of that seeding (the plan is the one for K).
+struct PlanFacts {
+    kpp_plan plan;
+    bool skips;    // its passes skip rows (kpp_pass.cuh)
+    size_t bytes;  // workspace it needs to run as planned
+};
+kpp_status plan_facts(int64_t N, int32_t d, int32_t K, kpp_dtype dtype, const kpp_options *opts,
+                      PlanFacts *out);
+kpp_status seed_passes(const void *points, const float *row_scales, int64_t N, int32_t d,
+                       int32_t K, int32_t passes, kpp_dtype dtype, uint64_t seed,
+                       uint64_t stream_id, const int64_t *forced_prefix, int32_t n_forced,
+                       int64_t *indices_out, float *d2_out, double *phi_out, void *workspace,
+                       size_t workspace_bytes, kpp_stream_t stream, const kpp_options *opts);
 
 } // namespace kpp
 

@@ -125,15 +125,17 @@ kpp_options make_opts(int form, int lanes, int ctas_per_sm, int smem_cache, int 
 }
 
 // The candidate grid: the small form (where the problem fits one SM), every
-// built lanes-per-row specialisation of the two other forms; for the persistent form with and without the shared-memory point cache and
-// three smallest row blocks per CTA, for the streamed form three grid sizes.
+// built lanes-per-row specialisation of the two other forms; for the persistent
+// form passes that skip rows or read every row, the latter with and without the
+// shared-memory point cache, and three smallest row blocks per CTA, for the
+// streamed form three grid sizes.
 std::vector<kpp_options> candidates()
 {
     static const int kLanes[] = {0, 1, 2, 4, 8, 16, 32};
     std::vector<kpp_options> c;
     c.push_back(make_opts(KPP_FORM_SMALL, 0, 0, 0, 0));
     for (int lanes : kLanes) {
-        for (int cache : {0, -1})
+        for (int cache : {0, -1, 1 << 30, -2})
             for (int min_rows : {0, 512, 8192})
                 c.push_back(make_opts(KPP_FORM_PERSISTENT, lanes, 0, cache, min_rows));
         for (int cps : {0, 2, 8})
@@ -143,12 +145,20 @@ std::vector<kpp_options> candidates()
 }
 
 // What distinguishes two candidates' launches (equal plans run the same code).
-std::tuple<int, int, int, int, int64_t, int64_t, int, int> signature(const kpp_plan &p,
-                                                                   const kpp_options &o)
+using Signature = std::tuple<int, int, int, int, int64_t, int64_t, bool, int, int>;
+Signature signature(const PlanFacts &f, const kpp_options &o)
 {
+    const kpp_plan &p = f.plan;
     return std::make_tuple(p.form, p.grid, p.lanes_per_row, p.d2_in_smem, p.rows_per_cta,
-                           p.cached_rows_per_cta, o.l2_policy, o.alternate);
+                           p.cached_rows_per_cta, f.skips, f.skips ? 0 : o.l2_policy, o.alternate);
 }
+
+// The fastest candidate of a kind so far.
+struct Best {
+    float ms = -1.f; // per pass
+    int order = 0;   // when it was tried
+    kpp_options o;
+};
 
 } // namespace
 
@@ -217,68 +227,68 @@ kpp_status kpp_tune(const void *points, const float *row_scales, int64_t N, int3
         return KPP_ERR_CUDA;
     }
     kpp_status result = KPP_OK;
-    float best_ms = -1.f;
-    kpp_options best;
-    std::memset(&best, 0, sizeof(best));
-    std::vector<std::tuple<int, int, int, int, int64_t, int64_t, int, int>> seen;
+    Best kind[2]; // plans that read every row; plans whose passes skip rows
+    int tried = 0;
+    std::vector<Signature> seen;
 
-    // one candidate: a warm-up run (it also captures a streamed graph), then
-    // two timed runs; ms per pass, or < 0 if the candidate does not apply
-    auto trial = [&](const kpp_options &o, float *ms) -> kpp_status {
+    // `passes` passes of the seeding under `o`: a warm-up run (it also captures a
+    // streamed graph), then `runs` timed runs; ms per pass, or < 0 if the
+    // candidate does not apply
+    auto time_passes = [&](const kpp_options &o, int32_t passes, bool warm, int runs,
+                           float *ms) -> kpp_status {
         *ms = -1.f;
-        kpp_plan plan;
-        if (kpp_describe(N, d, Kt, dtype, &o, &plan) != KPP_OK ||
-            (size_t)plan.workspace_bytes > workspace_bytes)
-            return KPP_OK;
-        const auto sig = signature(plan, o);
-        if (std::find(seen.begin(), seen.end(), sig) != seen.end())
-            return KPP_OK;
-        seen.push_back(sig);
-        kpp_status st = kpp_seed(points, row_scales, N, d, Kt, dtype, 1, 0, nullptr, 0,
-                                 indices_out, d2_out, nullptr, workspace, workspace_bytes, stream,
-                                 &o);
-        if (st != KPP_OK)
-            return st == KPP_ERR_INVALID_ARG || st == KPP_ERR_WORKSPACE ? st : KPP_OK;
-        st = kpp_read_status(workspace, stream);
-        if (st == KPP_ERR_DEGENERATE || st == KPP_ERR_CUDA)
-            return st; // the data or the device, not the candidate
-        if (st != KPP_OK)
-            return KPP_OK; // e.g. a bounded wait gave up: not a candidate
-        constexpr int kRuns = 2;
+        auto run = [&] {
+            return seed_passes(points, row_scales, N, d, K, passes, dtype, 1, 0, nullptr, 0,
+                               indices_out, d2_out, nullptr, workspace, workspace_bytes, stream,
+                               &o);
+        };
+        kpp_status st = KPP_OK;
+        if (warm) {
+            st = run();
+            if (st != KPP_OK)
+                return st == KPP_ERR_INVALID_ARG || st == KPP_ERR_WORKSPACE ? st : KPP_OK;
+            st = kpp_read_status(workspace, stream);
+            if (st == KPP_ERR_DEGENERATE || st == KPP_ERR_CUDA)
+                return st; // the data or the device, not the candidate
+            if (st != KPP_OK)
+                return KPP_OK; // e.g. a bounded wait gave up: not a candidate
+        }
         if (cudaEventRecord(e0, s) != cudaSuccess)
             return KPP_ERR_CUDA;
-        for (int r = 0; r < kRuns; ++r) {
-            st = kpp_seed(points, row_scales, N, d, Kt, dtype, 1, 0, nullptr, 0, indices_out,
-                          d2_out, nullptr, workspace, workspace_bytes, stream, &o);
-            if (st != KPP_OK)
+        for (int r = 0; r < runs; ++r)
+            if (run() != KPP_OK)
                 return KPP_OK;
-        }
         float t = 0.f;
         if (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
             cudaEventElapsedTime(&t, e0, e1) != cudaSuccess)
             return KPP_ERR_CUDA;
-        if (kpp_read_status(workspace, stream) != KPP_OK)
-            return KPP_OK;
-        *ms = t / (kRuns * Kt);
+        st = kpp_read_status(workspace, stream);
+        if (st == KPP_ERR_CUDA)
+            return st;
+        if (st == KPP_OK)
+            *ms = t / (runs * passes);
         return KPP_OK;
     };
-    bool best_skips = false;
+    // one candidate, against the best of its kind: a later one must win by more
+    // than 1 %, so that timing noise alone does not move the choice away from
+    // the earlier (default) ones
     auto consider = [&](const kpp_options &o) -> kpp_status {
+        PlanFacts f;
+        if (plan_facts(N, d, K, dtype, &o, &f) != KPP_OK || f.bytes > workspace_bytes)
+            return KPP_OK;
+        const Signature sig = signature(f, o);
+        if (std::find(seen.begin(), seen.end(), sig) != seen.end())
+            return KPP_OK;
+        seen.push_back(sig);
         float ms;
-        const kpp_status st = trial(o, &ms);
-        // a later candidate must win by more than 1 %: timing noise alone
-        // does not move the choice away from the earlier (default) ones.
-        // The trial's passes are a seeding's first ones, which can skip few
-        // rows; the later ones of a long seeding skip most (10^7 x 64,
-        // K = 1024: 0.39 ms falling to 0.03), so a plan that skips rows is
-        // worth a slower start.
-        const bool skips = Kt < K / 2 && plan_skips_rows(N, d, K, dtype, &o);
-        const float win = skips == best_skips ? 0.99f : (skips ? 1.25f : 0.8f);
-        if (st == KPP_OK && ms > 0.f && (best_ms < 0.f || ms < win * best_ms)) {
-            best_ms = ms;
-            best = o;
-            best_skips = skips;
+        const kpp_status st = time_passes(o, Kt, true, 2, &ms);
+        Best &b = kind[f.skips];
+        if (st == KPP_OK && ms > 0.f && (b.ms < 0.f || ms < 0.99f * b.ms)) {
+            b.ms = ms;
+            b.o = o;
+            b.order = tried;
         }
+        ++tried;
         return st;
     };
 
@@ -287,9 +297,12 @@ kpp_status kpp_tune(const void *points, const float *row_scales, int64_t N, int3
         if (result != KPP_OK)
             break;
     }
-    // refine the persistent winner's traversal and L2 policy
-    if (result == KPP_OK && best_ms > 0.f && best.form == KPP_FORM_PERSISTENT) {
-        const kpp_options base = best;
+    // refine the persistent winners' traversal and (where every row is read) L2 policy
+    for (Best &b : kind) {
+        if (result != KPP_OK || b.ms < 0.f || b.o.form != KPP_FORM_PERSISTENT)
+            continue;
+        const int order = b.order; // (a variant of the same plan)
+        const kpp_options base = b.o;
         for (int l2 : {-1, 2}) {
             kpp_options v = base;
             v.l2_policy = l2;
@@ -297,11 +310,40 @@ kpp_status kpp_tune(const void *points, const float *row_scales, int64_t N, int3
                 break;
         }
         if (result == KPP_OK) {
-            kpp_options v = best;
+            kpp_options v = b.o;
             v.alternate = -1;
             result = consider(v);
         }
+        b.order = order;
     }
+    // The kinds against each other: the first passes say little, since the share
+    // of the rows that a pass skips grows with the seeds chosen (10^7 x 64,
+    // K = 1024 in clusters: 0.39 ms a pass falling to 0.03) or not, as the data
+    // has it (2 10^6 x 64, K = 256 in clusters: 32 passes still favour the plan
+    // that reads every row, which takes 18.1 ms in all for 8.9).  So each of the
+    // two winners takes a whole seeding.
+    int win = kind[1].ms > 0.f && (kind[0].ms < 0.f || kind[1].order < kind[0].order) ? 1 : 0;
+    if (result == KPP_OK && kind[0].ms > 0.f && kind[1].ms > 0.f) {
+        float ms[2] = {kind[0].ms, kind[1].ms};
+        for (int k = 0; K > Kt && k < 2; ++k) {
+            float t;
+            const kpp_status st =
+                time_passes(kind[k].o, K, kind[k].o.form == KPP_FORM_STREAMED, 1, &t);
+            if (st == KPP_ERR_CUDA)
+                result = st;
+            // (fewer distinct points than K: the first passes decide)
+            if (st != KPP_OK || t < 0.f) {
+                ms[0] = kind[0].ms;
+                ms[1] = kind[1].ms;
+                break;
+            }
+            ms[k] = t;
+        }
+        if (ms[1 - win] < 0.99f * ms[win])
+            win = 1 - win;
+    }
+    const kpp_options best = kind[win].o;
+    const float best_ms = kind[win].ms;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (result != KPP_OK)

@@ -1,0 +1,74 @@
+"""The autotuner between plans whose passes skip rows and plans that read every
+row: on data without clusters, where nothing can be skipped, its choice is not
+slower than the plan that reads every row; on clusters not slower than the
+automatic one, however few passes it may time."""
+import pytest
+import torch
+
+import paper_1908_02136_gb300 as kpp
+from paper_1908_02136_gb300 import datagen
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda:0"
+
+
+@pytest.fixture(autouse=True)
+def clean_table():
+    kpp.kpp_tune_clear()
+    yield
+    kpp.kpp_tune_clear()
+
+
+def _ms(x, K, opts):
+    N, d = x.shape
+    with torch.cuda.device(DEV):
+        ws = kpp.workspace_for(N, d, K, kpp.F32, x.device, opts)
+    out = kpp.seed(x, K, 3, opts=opts, workspace=ws)
+    best = float("inf")
+    for _ in range(4):
+        a, b = torch.cuda.Event(True), torch.cuda.Event(True)
+        a.record()
+        kpp.seed(x, K, 3, opts=opts, workspace=ws, out=out, check=False)
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b))
+    return best
+
+
+@pytest.mark.parametrize("passes", [4, 16])
+def test_choice_on_data_without_clusters(passes):
+    N, d, K = 2_000_000, 64, 96
+    x = torch.randn(N, d, device=DEV)
+    best, _ = kpp.tune(x, K, passes=passes)
+    plain = _ms(x, K, {"form": kpp.FORM_PERSISTENT, "smem_cache": 1 << 30})
+    # the tuner's own margin is 1 %, runs of one plan differ by another
+    assert _ms(x, K, best) <= 1.03 * plain
+
+
+@pytest.mark.parametrize("passes", [4, 16])
+def test_choice_on_clusters(passes):
+    N, d, K = 2_000_000, 64, 256
+    x = torch.from_numpy(datagen.gmm(N, d, K, seed=1)).to(DEV)
+    auto = _ms(x, K, None)
+    best, _ = kpp.tune(x, K, passes=passes)
+    assert _ms(x, K, best) <= 1.03 * auto
+
+
+def test_workspace_without_labels_times_plans_that_read_every_row():
+    """A workspace that cannot hold the labels skips the plans that keep them."""
+    import ctypes
+
+    N, d, K = 2_000_000, 64, 64
+    x = torch.from_numpy(datagen.gmm(N, d, K, seed=2)).to(DEV)
+    idx = torch.empty(K, dtype=torch.int64, device=DEV)
+    d2 = torch.empty(N, dtype=torch.float32, device=DEV)
+    ws = torch.empty(1 << 20, dtype=torch.uint8, device=DEV)
+    best = kpp.Options()
+    with torch.cuda.device(DEV):
+        st = kpp.kpp_tune(x.data_ptr(), None, N, d, K, kpp.F32, idx.data_ptr(), d2.data_ptr(),
+                          ws.data_ptr(), ws.numel(),
+                          ctypes.c_void_p(torch.cuda.current_stream().cuda_stream), 8, best)
+        assert st == kpp.OK
+        opts = {f: getattr(best, f) for f, _ in kpp.Options._fields_ if f != "reserved"}
+        assert kpp.kpp_workspace_size(N, d, K, kpp.F32, opts) <= ws.numel()
