@@ -318,7 +318,9 @@ KPP_API kpp_status kpp_seed_batched(const kpp_problem *problems, int32_t n, kpp_
  *                                        (their contents are undefined after)
  *   workspace   >= kpp_tune_workspace_size(N, d, K, dtype) bytes covers every
  *               candidate; a smaller one skips the candidates it cannot hold
- *   best_out    host: the winning options (form never KPP_FORM_AUTO)
+ *   best_out    host: the winning options (form KPP_FORM_AUTO only for the
+ *               persistent kernel of a d without a specialisation, which no
+ *               form names)
  *   best_ms_per_pass  host, may be NULL: the winner's mean time per pass of
  *               the first min(K, passes)
  * Blocks the calling thread (it synchronises `stream`).  The winner is also

@@ -313,15 +313,9 @@ kpp_status make_plan(int64_t N, int32_t d, int32_t K, int dt, const kpp_options 
     std::memset(&o, 0, sizeof(o));
     if (opts)
         o = *opts;
-    // The autotuner's choice for this shape.  (It times the forms a caller
-    // can name; for a d without a specialisation that leaves the streamed one,
-    // behind the automatic choice.)
     kpp_options tuned;
-    PersistentKernel named;
-    if (tuned_options(N, d, K, dt, o, &tuned) &&
-        (tuned.form != KPP_FORM_STREAMED || !any_d_rule(d, K, dt) ||
-         persistent_lookup(dt, d, 0, false, &named)))
-        o = tuned;
+    if (tuned_options(N, d, K, dt, o, &tuned))
+        o = tuned; // the autotuner's choice for this shape
     const int sms = device_sms();
     if (sms <= 0)
         return KPP_ERR_CUDA;

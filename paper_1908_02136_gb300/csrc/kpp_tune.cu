@@ -128,7 +128,10 @@ kpp_options make_opts(int form, int lanes, int ctas_per_sm, int smem_cache, int 
 // built lanes-per-row specialisation of the two other forms; for the persistent
 // form passes that skip rows or read every row, the latter with and without the
 // shared-memory point cache, and three smallest row blocks per CTA, for the
-// streamed form three grid sizes.
+// streamed form three grid sizes.  Last the automatic choice where that is the
+// persistent any-d kernel, which no form names (`consider` passes it over
+// elsewhere): one CTA per SM, what that kernel runs, keeps it from being looked
+// up among the recorded choices.
 std::vector<kpp_options> candidates()
 {
     static const int kLanes[] = {0, 1, 2, 4, 8, 16, 32};
@@ -141,6 +144,7 @@ std::vector<kpp_options> candidates()
         for (int cps : {0, 2, 8})
             c.push_back(make_opts(KPP_FORM_STREAMED, lanes, cps, 0, 0));
     }
+    c.push_back(make_opts(KPP_FORM_AUTO, 0, 1, 0, 0));
     return c;
 }
 
@@ -275,6 +279,9 @@ kpp_status kpp_tune(const void *points, const float *row_scales, int64_t N, int3
     auto consider = [&](const kpp_options &o) -> kpp_status {
         PlanFacts f;
         if (plan_facts(N, d, K, dtype, &o, &f) != KPP_OK || f.bytes > workspace_bytes)
+            return KPP_OK;
+        if (o.form == KPP_FORM_AUTO &&
+            !(f.plan.form == KPP_FORM_PERSISTENT && f.plan.lanes_per_row == 0))
             return KPP_OK;
         const Signature sig = signature(f, o);
         if (std::find(seen.begin(), seen.end(), sig) != seen.end())

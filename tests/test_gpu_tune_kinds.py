@@ -72,3 +72,46 @@ def test_workspace_without_labels_times_plans_that_read_every_row():
         assert st == kpp.OK
         opts = {f: getattr(best, f) for f, _ in kpp.Options._fields_ if f != "reserved"}
         assert kpp.kpp_workspace_size(N, d, K, kpp.F32, opts) <= ws.numel()
+
+
+@pytest.mark.parametrize("N,d,K,dtype", [(100_003, 50, 64, "f32"), (200_003, 100, 20, "bf16")])
+def test_any_d_is_timed_recorded_and_returned(N, d, K, dtype):
+    """The persistent any-d kernel, which no form names, takes part: what the
+    tuner returns and records is what later automatic calls run."""
+    code = {"f32": kpp.F32, "bf16": kpp.BF16}[dtype]
+    x = torch.from_numpy(datagen.gmm(N, d, K, seed=d)).to(DEV)
+    if dtype == "bf16":
+        x = kpp.quantize(x, dtype)
+    ref = kpp.seed(x, K, 3, opts={"form": kpp.FORM_STREAMED})
+    for _ in range(2):  # a recorded choice does not stand in for the automatic one
+        best, ms = kpp.tune(x, K, passes=8)
+        with torch.cuda.device(DEV):
+            st, plan = kpp.kpp_describe(N, d, K, code, best)
+            assert st == kpp.OK
+            assert plan.form == kpp.FORM_PERSISTENT and plan.lanes_per_row == 0 and ms > 0
+            st, auto = kpp.kpp_describe(N, d, K, code)
+            assert st == kpp.OK and auto.as_dict() == plan.as_dict()
+    for opts in (best, None):
+        out = kpp.seed(x, K, 3, opts=opts)
+        assert torch.equal(ref[0], out[0]) and torch.equal(ref[1], out[1])
+
+
+def test_a_recorded_streamed_choice_stands_for_any_d(tmp_path):
+    """A line of the cache file for a d without a specialisation is used as it is."""
+    import json
+    import os
+    import subprocess
+    import sys
+
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    N, d, K = 100_003, 50, 64
+    p = torch.cuda.get_device_properties(0)
+    cache = tmp_path / "tune.txt"
+    cache.write_text(f"kpp-tune 1 {p.name.replace(' ', '_')}/{p.multi_processor_count} 0 {d} {N} {K} "
+                     f"{kpp.FORM_STREAMED} 0 2 0 0 0 0\n")
+    code = ("import json, torch, paper_1908_02136_gb300 as kpp; torch.zeros(1, device='cuda:0');"
+            f"st, p = kpp.kpp_describe({N}, {d}, {K}, kpp.F32); print(json.dumps([st, p.form]))")
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=root,
+                       env=dict(os.environ, KPP_TUNE_CACHE=str(cache)), timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert json.loads(r.stdout.strip().splitlines()[-1]) == [kpp.OK, kpp.FORM_STREAMED]
