@@ -830,7 +830,8 @@ def roofline_for(plan, form_name, N, d, K, eb, has_scales, ms_per_step, wl_name,
     L2 read rate for L2, with the live pure-read rates reported beside."""
     peaks = measured_peaks()
     hbm_copy = peaks["hbm_gbs"] if peaks else 6800.0
-    launches = plan["launches"]
+    # (a second launch of the persistent form stands by: one runs all passes)
+    launches = 1 if form_name == "persistent" else plan["launches"]
     per_launch_ms = ms_per_step / launches
     passes_per_launch = K // launches
     point_bytes = N * d * eb + (4 * N if has_scales else 0)

@@ -142,7 +142,9 @@ typedef struct {
     int32_t form;                /* kpp_form actually chosen */
     int32_t grid;                /* CTAs per launch */
     int32_t threads;             /* threads per CTA */
-    int32_t launches;            /* kernel launches per seeding */
+    int32_t launches;            /* kernel launches per seeding (persistent form: 2 where
+                                    the kernel that reads every row stands by in case
+                                    passes find next to none to skip) */
     int32_t lanes_per_row;       /* 0 for the generic (any d) kernel */
     int32_t d2_in_smem;          /* persistent form: D^2 held in shared memory */
     int64_t rows_per_cta;        /* contiguous row block of each CTA */

@@ -17,6 +17,7 @@ constexpr size_t kAlign = 256;
 constexpr int kMaxDim = 4096;
 constexpr int kDefaultCtasPerSm = 4;
 constexpr int kPruneMinK = 8; // fewer passes than this read every row
+constexpr double kHandBytes = 20e9; // of rows in all passes: from here on the plain kernel stands by
 
 size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -45,6 +46,10 @@ struct Plan {
     int nseg;   // segments (warps) per block
     int64_t sw; // rows per super-iteration
     bool prune; // persistent form: passes skip the rows they cannot change
+    // the plain kernel to go on where they skip next to none (null: none)
+    const void *hand_fn;
+    size_t hand_smem;
+    int64_t hand_supers; // its point cache
     // workspace layout (byte offsets after the control block)
     size_t off_bsum, off_seg, off_slots;
     size_t min_bytes;   // without the labels of `prune` (a workspace that holds no
@@ -96,6 +101,7 @@ kpp_status plan_streamed(int64_t N, int32_t d, int dt, const kpp_options &o, int
     chunk = (chunk + a - 1) / a * a;
     pl->form = KPP_FORM_STREAMED;
     pl->prune = false;
+    pl->hand_fn = nullptr;
     pl->chunk = chunk;
     pl->nblocks = (int)((N + chunk - 1) / chunk);
     pl->grid = pl->nblocks;
@@ -135,6 +141,7 @@ kpp_status plan_small(int64_t N, int32_t d, int dt, Plan *pl)
     pl->nseg = small_threads() / 32;
     pl->sw = 1;
     pl->prune = false;
+    pl->hand_fn = nullptr;
     pl->off_bsum = pl->off_seg = pl->off_slots = sizeof(Control);
     pl->label_bytes = 0;
     pl->min_bytes = pl->ws_bytes = sizeof(Control);
@@ -193,7 +200,8 @@ kpp_status plan_persistent_at(int64_t N, int32_t d, int32_t K, int dt, const kpp
     cudaFuncAttributes fa;
     if (cudaFuncGetAttributes(&fa, any_d ? pl->pk.prune_smem : pl->pk.fn_smem) != cudaSuccess)
         return KPP_ERR_CUDA;
-    const int64_t budget = ((int64_t)optin - (int64_t)fa.sharedSizeBytes - 1024) / per_sm;
+    const int most = optin - (int)fa.sharedSizeBytes - 1024; // static sizes differ a little
+    const int64_t budget = (int64_t)most / per_sm;
     int64_t used = 0;
     // D^2 of the block and its 32-row chunk sums
     const int64_t d2_bytes = ((4 * chunk + 15) & ~15ll) + 8 * ((chunk + 31) / 32);
@@ -216,6 +224,9 @@ kpp_status plan_persistent_at(int64_t N, int32_t d, int32_t K, int dt, const kpp
             supers = 0;
     }
     pl->psmem = (size_t)(supers * unit + (d2_in_smem ? d2_bytes : 0));
+    const bool plain_in_smem = d2_in_smem;
+    const int64_t plain_supers = supers;
+    const size_t plain_smem = pl->psmem;
     // Passes that skip rows, unless the caller asked for a point cache or half
     // of the block fits one (6 020 x 64 BF16, K = 993: 7.3 ms with 80 % of the
     // rows cached, 8.7 skipping; 100 000 x 64 FP32, K = 100, 40 %: 968 / 842 us).
@@ -255,6 +266,21 @@ kpp_status plan_persistent_at(int64_t N, int32_t d, int32_t K, int dt, const kpp
     } else if (any_d) {
         return KPP_ERR_UNSUPPORTED;
     }
+    // D^2 left shared memory for the lists: the plain kernel stands by where its
+    // launch is a small part of the seeding (20 GB of rows take 3 ms).  Narrow
+    // rows gain from the row pipe even where none is skipped (4 10^6 x 16, K = 256
+    // 12.2 / 10.8 ms, x 8 BF16 4.8 / 3.8).
+    pl->hand_fn = nullptr;
+    if (pl->prune && !any_d && plain_in_smem && !d2_in_smem &&
+        pl->pk.row_bytes >= kHandRowBytes &&
+        (double)N * pl->pk.row_bytes * K >= kHandBytes) {
+        pl->hand_fn = pl->pk.fn_smem;
+        pl->hand_smem = plain_smem;
+        pl->hand_supers = plain_supers;
+        if (cudaFuncSetAttribute(pl->hand_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most) !=
+            cudaSuccess)
+            return KPP_ERR_CUDA;
+    }
     if (pl->prune || any_d)
         pl->pfn = d2_in_smem ? pl->pk.prune_smem : pl->pk.prune_global;
     else
@@ -262,8 +288,8 @@ kpp_status plan_persistent_at(int64_t N, int32_t d, int32_t K, int dt, const kpp
     // static + dynamic shared memory above 48 KB needs the opt-in attribute.  It
     // belongs to the kernel, not to the call: always the same value, or another
     // thread's smaller plan would have this one's launch refused.
-    if (cudaFuncSetAttribute(pl->pfn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             optin - (int)fa.sharedSizeBytes) != cudaSuccess)
+    if (cudaFuncSetAttribute(pl->pfn, cudaFuncAttributeMaxDynamicSharedMemorySize, most) !=
+        cudaSuccess)
         return KPP_ERR_CUDA;
     int resident = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, pl->pfn, persistent_threads(),
@@ -397,7 +423,16 @@ kpp_status run_persistent(const Plan &pl, const Problem &p, cudaStream_t stream)
     // never carries the tag a pass waits for
     if (cudaMemsetAsync(p.ctl, 0, pl.min_bytes, stream) != cudaSuccess)
         return KPP_ERR_CUDA;
-    return persistent_launch(pl.pfn, pl.grid, pl.psmem, p, pl.pargs, stream) == cudaSuccess
+    if (persistent_launch(pl.pfn, pl.grid, pl.psmem, p, pl.pargs, stream) != cudaSuccess)
+        return KPP_ERR_LAUNCH;
+    if (!pl.hand_fn)
+        return KPP_OK;
+    Problem rest = p;
+    rest.prune = 0;
+    rest.hand_from = kTakeOver;
+    PersistArgs args = pl.pargs;
+    args.cache_supers = pl.hand_supers;
+    return persistent_launch(pl.hand_fn, pl.grid, pl.hand_smem, rest, args, stream) == cudaSuccess
                ? KPP_OK
                : KPP_ERR_LAUNCH;
 }
@@ -462,6 +497,16 @@ kpp_status run_streamed(const Plan &pl, const Problem &p, cudaStream_t stream, i
 
 bool aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
+// The pass that decides on a hand-over: about a sixteenth of the seeds, a pass
+// in which every CTA tests its rows, no earlier than the second such.
+int32_t hand_pass(int32_t K)
+{
+    const int32_t most = 128; // (the bounds stay a small part of a block: 4 m <= rows)
+    int32_t n = K / 16 / kPruneProbe;
+    n = n < 1 ? 1 : (n > most ? most : n);
+    return n * kPruneProbe + 1;
+}
+
 // What a plan looks like from outside.
 void fill_plan(const Plan &pl, int64_t N, int32_t d, int32_t K, kpp_plan *plan)
 {
@@ -479,7 +524,7 @@ void fill_plan(const Plan &pl, int64_t N, int32_t d, int32_t K, kpp_plan *plan)
         plan->smem_bytes = (int64_t)pl.psmem;
     } else if (pl.form == KPP_FORM_PERSISTENT) {
         plan->threads = persistent_threads();
-        plan->launches = 1;
+        plan->launches = pl.hand_fn ? 2 : 1;
         plan->lanes_per_row = pl.pk.lanes;
         plan->d2_in_smem = pl.pfn == pl.pk.fn_smem || pl.pfn == pl.pk.prune_smem ? 1 : 0;
         plan->cached_rows_per_cta = pl.pargs.cache_supers * pl.nseg * pl.sw;
@@ -561,6 +606,7 @@ kpp_status seed_passes(const void *points, const float *row_scales, int64_t N, i
         p.slots = reinterpret_cast<unsigned long long *>(ws + pl.off_slots);
         p.mail = &p.ctl->mail;
         p.prune = pl.prune ? 1 : 0;
+        p.hand_from = pl.hand_fn ? hand_pass(K) : 0;
         p.labels = reinterpret_cast<uint16_t *>(ws + pl.min_bytes);
     } else {
         p.block_sums = reinterpret_cast<float2 *>(ws + pl.off_bsum);

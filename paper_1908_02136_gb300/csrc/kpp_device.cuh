@@ -24,7 +24,10 @@ struct Control {
     unsigned long long mail; // persistent form: (drawn index << 32) | (pass + 1)
     uint32_t timeout_where;  // persistent form: pass whose wait gave up
     uint32_t bounds_site;    // debug build: site of the first index out of bounds
-    uint32_t pad_[58];
+    unsigned long long skipped; // persistent form: rows left unread by the pass that
+                                //   decides on the hand-over (kpp_persistent.cuh)
+    int32_t hand_pass;          //   the pass from which plain passes go on, or 0
+    uint32_t pad_[55];
 };
 
 // ---------------------------------------------------------------------------
@@ -55,6 +58,8 @@ __device__ __forceinline__ bool kpp_check(Control *ctl, bool ok, uint32_t site)
 constexpr int kSlotWords = 4;
 static_assert(sizeof(Control) == 256, "control block is 256 bytes");
 
+constexpr int32_t kTakeOver = -1; // Problem::hand_from
+
 // Everything a seeding kernel needs about one problem.
 struct Problem {
     const void *points;
@@ -81,6 +86,10 @@ struct Problem {
     int32_t recompute;         // streamed form: every pass rebuilds D^2 from all chosen seeds
     int32_t exact_draws;       // every draw decision in FP64 (the near-tie path), for testing
     int32_t prune;             // persistent form: skip the rows that a pass cannot change
+    int32_t hand_from;         //   > 0: the pass after which it hands over to the plain
+                               //   kernel if next to no row was skipped; kTakeOver: this is
+                               //   that kernel.  (Here, in what was padding: a larger struct
+                               //   costs the batched kernel, which reads it from memory, 1 %)
     uint16_t *labels;          //   their nearest centres [N] (D^2 in the output array only)
     // point-sharded seeding (one contiguous row range of a larger problem):
     // the centre of the pass comes from the exchange buffer `xchg` (global

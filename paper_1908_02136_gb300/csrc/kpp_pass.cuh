@@ -577,6 +577,8 @@ __device__ __forceinline__ Pair pass_rows(const PassIO &io, const CentreRegs<DT,
 // ---------------------------------------------------------------------------
 constexpr int kPruneCentres = 2048; // centres with a bound; rows of later ones are always read
 constexpr uint16_t kNoLabel = 0xffff;
+constexpr int kPruneProbe = 8; // every so many passes look again for rows to skip
+constexpr int kHandRowBytes = 128; // rows from which passes that skip none hand over
 
 // Largest D^2 of a row of centre a that centre c at squared distance s2 from
 // a cannot lower (negative: none).

@@ -59,12 +59,33 @@ struct BlockShared {
     int few;                   // they were few enough to go on skipping
 };
 
+// Where plain passes go on (below): from pass `pass` (0: nowhere), whose centre is
+// row ci.
+struct HandOver {
+    int pass;
+    int64_t ci;
+};
+
 // Passes test for rows to skip while the rows read, the chosen centres' (for
 // their bounds) included, were at most kPruneKeep of the block's; above that
 // they read every row, and every kPruneProbe-th pass tests again as long as the
 // bounds are a small part of it.
 constexpr float kPruneKeep = 0.8f;
-constexpr int kPruneProbe = 8;
+
+// Hand-over.  Where the lists push D^2 out of shared memory, passes over data
+// without clusters, where no row is ever skipped, pay for it (4 10^6 x 32,
+// K = 256 18.6 -> 20.2 ms).  There, in pass p.hand_from (a testing one, about a
+// sixteenth of the seeds: in clusters it skips the points of those that have a
+// seed, some sixteenth of all), every CTA adds the rows it skipped to
+// Control::skipped before it publishes its block sum, so that after the wait for
+// the sums every CTA reads the same total.  If it is under 1 / kHandOver of the
+// points, the kernel ends and the plain one, launched behind it, goes on with the
+// same blocks and exchange words, D^2 taken into shared memory (18.9 ms).  That
+// one pass's atomics and fences take 2.4 us; the second launch, where it finds
+// nothing to do, some 45 us of the call, whatever its grid and shared memory.
+// Plain passes inside this kernel instead gained nothing (20.6 ms): beside its
+// shared memory their loads have 28 KB of L1.
+constexpr int kHandOver = 50;
 
 // The seeding of problem p by a team of p.nblocks co-resident CTAs, this CTA
 // being member b: p.slots and p.mail are the team's own exchange words.
@@ -73,12 +94,17 @@ constexpr int kPruneProbe = 8;
 // seeding is done, or early -- the same way on every member -- on an error
 // recorded in the status word.
 // PRUNE: built with the passes that skip rows (p.prune turns them on); without
-// it the kernel is the plain one, its pass inline.
-template <int DT, int D, int L, int MODE, bool PRUNE>
-__device__ __forceinline__ void seed_blocks(const Problem &p, const PersistArgs &a, const int b,
-                                            char *smem, BlockShared &sh)
+// it the kernel is the plain one, its pass inline.  SPLIT: built to hand over
+// (PRUNE; `hand` is a shared word) or to take over, at `from`; the code costs
+// kernels that never do up to 2 %.
+template <int DT, int D, int L, int MODE, bool PRUNE, bool SPLIT = false>
+__device__ __forceinline__ HandOver seed_blocks(const Problem &p, const PersistArgs &a, const int b,
+                                            char *smem, BlockShared &sh,
+                                            int *hand = nullptr, const HandOver from = HandOver{})
 {
     using G = Geom<DT, D, L>;
+    constexpr bool kHands = SPLIT && PRUNE;
+    constexpr bool kTakes = SPLIT && !PRUNE;
     float2 *segsum = sh.segsum;
     DrawShared &ds = sh.ds;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -106,8 +132,11 @@ __device__ __forceinline__ void seed_blocks(const Problem &p, const PersistArgs 
                           D == 0 ? generic_centre_floats(DT, p.d) : 0);
     float *thr = reinterpret_cast<float *>(smem + pl.thr);
     int32_t *cidx = reinterpret_cast<int32_t *>(smem + pl.cidx);
-    if (threadIdx.x == 0)
+    if (threadIdx.x == 0) {
         sh.few = 0;
+        if (kHands)
+            *hand = 0;
+    }
 
     // the plan's limits: this block exists, the level-1 stage and the chunk
     // sums hold what the draw will put there (every CTA sees the same values)
@@ -115,21 +144,28 @@ __device__ __forceinline__ void seed_blocks(const Problem &p, const PersistArgs 
                    b >= 0 && b < p.nblocks && p.nblocks <= kMaxBlocks && r0 < r1 &&
                        (!chunk_path || nchunks <= kMaxChunks),
                    201))
-        return;
-    int64_t ci = first_seed(p);
+        return HandOver{};
+    const int m0 = kTakes ? from.pass : 0; // the first pass here
+    int64_t ci = kTakes && m0 > 0 ? from.ci : first_seed(p);
     if (ci < 0 || ci >= p.N) {
         if (b == 0 && threadIdx.x == 0)
             atomicCAS(&p.ctl->status, KPP_OK, KPP_ERR_INVALID_ARG);
-        return; // every CTA takes this branch: nobody is left waiting
+        return HandOver{}; // every CTA takes this branch: nobody is left waiting
     }
     if (threadIdx.x == 0) {
-        if (b == 0)
+        if (b == 0 && m0 == 0)
             p.idx[0] = ci;
-        if (p.K > 1)
-            ds.th[1] = thresh_for_u(philox_uniform(p.seed, p.stream_id, 1), p.exact_draws);
+        if (m0 + 1 < p.K)
+            ds.th[(m0 + 1) & 1] =
+                thresh_for_u(philox_uniform(p.seed, p.stream_id, (uint64_t)(m0 + 1)), p.exact_draws);
+    }
+    if (kTakes && m0 > 0) {
+        for (int64_t r = r0 + threadIdx.x; r < r1; r += blockDim.x)
+            d2s[r - r0] = p.d2[r];
+        __syncthreads();
     }
 
-    for (int m = 0; m < p.K; ++m) {
+    for (int m = m0; m < p.K; ++m) {
         const bool last = (m == p.K - 1);
         const int next = m + 1;
 
@@ -143,7 +179,7 @@ __device__ __forceinline__ void seed_blocks(const Problem &p, const PersistArgs 
         io.scales = p.scales;
         io.cache = cache;
         io.cache_supers = a.cache_supers;
-        io.fill_cache = (m == 0);
+        io.fill_cache = (m == m0);
         io.d2 = p.d2;
         io.d2_out = last ? p.d2 : nullptr;
         io.d2s = d2s;
@@ -181,16 +217,24 @@ __device__ __forceinline__ void seed_blocks(const Problem &p, const PersistArgs 
 
         // publish this block's pair sum (segments in warp order)
         unsigned long long *slots = p.slots + (size_t)(m & 1) * p.nblocks * kSlotWords;
+        const bool counted = kHands && m > 0 && m == p.hand_from;
         if (threadIdx.x == 0) {
             Pair bs{};
             for (int w = 0; w < kPersistWarps; ++w)
                 bs.add(Pair{segsum[w].x, segsum[w].y});
+            if (counted && prune) {
+                int64_t skipped = r1 - r0;
+                for (int w = 0; w < kPersistWarps; ++w)
+                    skipped -= sh.active[w];
+                atomicAdd(&p.ctl->skipped, (unsigned long long)skipped);
+                __threadfence(); // before this block's sum, which everyone waits for
+            }
             st_relaxed_u64(slots + (size_t)b * kSlotWords, pack_slot(bs, m));
             if (p.nblocks == 1) // alone: this block's sum is level 1
                 ds.stage_pairs[0] = make_float2(bs.hi, bs.lo);
         }
         if (last && b != 0)
-            return; // only block 0 waits, to sum phi
+            return HandOver{}; // only block 0 waits, to sum phi
         const bool forced = !last && next < p.n_forced;
 
         if (warp == 0) {
@@ -203,6 +247,10 @@ __device__ __forceinline__ void seed_blocks(const Problem &p, const PersistArgs 
                                      ds.stage_pairs + k0);
             }
             __syncwarp();
+            if (counted && ok && lane == 0) {
+                __threadfence();
+                *hand = ld_relaxed_u64(&p.ctl->skipped) * kHandOver < (unsigned long long)p.N;
+            }
             if (ok && last) { // block 0: phi = the ordered sum of the final block sums
                 const PFind r = warp_pfind(
                     p.nblocks,
@@ -260,16 +308,18 @@ __device__ __forceinline__ void seed_blocks(const Problem &p, const PersistArgs 
         }
         __syncthreads();
         if (!ds.ok || last)
-            return;
+            return HandOver{};
         if (forced) {
             ci = p.forced[next];
             if (ci < 0 || ci >= p.N) {
                 if (b == 0 && threadIdx.x == 0)
                     atomicCAS(&p.ctl->status, KPP_OK, KPP_ERR_INVALID_ARG);
-                return; // the same forced index on every CTA
+                return HandOver{}; // the same forced index on every CTA
             }
             if (b == 0 && threadIdx.x == 0)
                 p.idx[next] = ci;
+            if (kHands && *hand)
+                return HandOver{next, ci};
             continue;
         }
         const int64_t owner = ds.owner;
@@ -286,7 +336,7 @@ __device__ __forceinline__ void seed_blocks(const Problem &p, const PersistArgs 
                     p.phi[0] = 0.0;
                 atomicCAS(&p.ctl->status, KPP_OK, KPP_ERR_DEGENERATE);
             }
-            return;
+            return HandOver{};
         }
 
         if (owner == b) {
@@ -394,8 +444,11 @@ __device__ __forceinline__ void seed_blocks(const Problem &p, const PersistArgs 
         __syncthreads();
         ci = ds.pick;
         if (ci < 0)
-            return; // a wait gave up: the status word says why
+            return HandOver{}; // a wait gave up: the status word says why
+        if (kHands && *hand)
+            return HandOver{next, ci}; // (on every CTA)
     }
+    return HandOver{};
 }
 
 template <int DT, int D, int L, int MODE, bool PRUNE>
@@ -404,7 +457,25 @@ __global__ void __launch_bounds__(kPersistThreads, 1)
 {
     extern __shared__ __align__(128) char smem[];
     __shared__ BlockShared sh;
-    seed_blocks<DT, D, L, MODE, PRUNE>(p, a, blockIdx.x, smem, sh);
+    constexpr bool kWide = Geom<DT, D, L>::RB >= kHandRowBytes;
+    if constexpr (PRUNE && MODE == D2_INPLACE && kWide) {
+        __shared__ int hand;
+        const HandOver h =
+            seed_blocks<DT, D, L, MODE, PRUNE, true>(p, a, blockIdx.x, smem, sh, &hand);
+        if (h.pass > 0 && blockIdx.x == 0 && threadIdx.x == 0)
+            p.ctl->hand_pass = h.pass;
+    } else if constexpr (!PRUNE && MODE == D2_SMEM && kWide) {
+        HandOver from{};
+        if (p.hand_from == kTakeOver) {
+            from.pass = p.ctl->hand_pass;
+            if (from.pass <= 0 || from.pass >= p.K)
+                return; // (on every CTA)
+            from.ci = p.idx[from.pass];
+        }
+        seed_blocks<DT, D, L, MODE, PRUNE, true>(p, a, blockIdx.x, smem, sh, nullptr, from);
+    } else {
+        seed_blocks<DT, D, L, MODE, PRUNE>(p, a, blockIdx.x, smem, sh);
+    }
 }
 
 // One specialisation of the persistent kernel, as listed by the per-dtype
