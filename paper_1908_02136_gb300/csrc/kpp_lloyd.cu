@@ -1085,7 +1085,7 @@ __global__ void __launch_bounds__(kOrdThreads)
 // perm[position] = point, positions grouped by label.
 __global__ void __launch_bounds__(kOrdThreads)
     lloyd_order_kernel(const int32_t *labels, int64_t N, int K, const int32_t *base,
-                       const int32_t *start, int32_t *perm)
+                       const int32_t *start, int32_t *perm, Control *ctl)
 {
     extern __shared__ int s_at[]; // [K] next position of this range's points
     const int t = threadIdx.x;
@@ -1102,8 +1102,11 @@ __global__ void __launch_bounds__(kOrdThreads)
             l[u] = i0 + u * kOrdThreads < hi ? label_at(labels, i0 + u * kOrdThreads, K) : -1;
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-            if (l[u] >= 0)
-                perm[atomicAdd(s_at + l[u], 1)] = (int32_t)(i0 + u * kOrdThreads);
+            if (l[u] >= 0) {
+                const int at = atomicAdd(s_at + l[u], 1);
+                if (kpp_check(ctl, at >= 0 && at < N, 511))
+                    perm[at] = (int32_t)(i0 + u * kOrdThreads);
+            }
     }
 }
 
@@ -1122,7 +1125,7 @@ __global__ void __launch_bounds__(kSegThreads, kSegCtas)
     lloyd_segment_kernel(const float *__restrict__ x, int64_t N, int d, int K,
                          const float *__restrict__ c, const int32_t *__restrict__ perm,
                          const int32_t *__restrict__ start, float *d2_out, double *sums,
-                         double *partial)
+                         double *partial, Control *ctl)
 {
     constexpr int RPS = 32 / LD; // rows per step
     extern __shared__ int s_start[]; // [K + 1]
@@ -1162,7 +1165,9 @@ __global__ void __launch_bounds__(kSegThreads, kSegCtas)
 #pragma unroll
                 for (int q = 0; q < ROWS; ++q) {
                     const int64_t at = p + q * RPS + sub;
-                    row[q] = at < e ? perm[at] : -1;
+                    row[q] = at < e && kpp_check(ctl, at >= 0 && at < N, 512) ? perm[at] : -1;
+                    if (!kpp_check(ctl, row[q] < N, 513))
+                        row[q] = -1;
                 }
                 float xv[ROWS][VEC];
 #pragma unroll
@@ -1270,7 +1275,7 @@ bool update_ordered(int64_t N, int d, int K)
 }
 
 using SegmentFn = void (*)(const float *, int64_t, int, int, const float *, const int32_t *,
-                           const int32_t *, float *, double *, double *);
+                           const int32_t *, float *, double *, double *, Control *);
 
 // Lanes per row by d, so that few lanes idle; 64 rows' worth of loads or 8 KB
 // a warp in flight.
@@ -1632,12 +1637,14 @@ kpp_status kpp_lloyd_step(const float *points, int64_t N, int32_t d, const float
         const size_t osmem = (size_t)K * 4;
         lloyd_count_kernel<<<octas, kOrdThreads, osmem, s>>>(labels_out, N, K, counts, base, start,
                                                              ticket);
-        lloyd_order_kernel<<<octas, kOrdThreads, osmem, s>>>(labels_out, N, K, base, start, perm);
+        lloyd_order_kernel<<<octas, kOrdThreads, osmem, s>>>(labels_out, N, K, base, start, perm,
+                                                             reinterpret_cast<Control *>(ws));
         // a full wave; fewer CTAs where a warp would get less than two batches
         const int64_t most = (N + 32 * (kSegThreads / 32) - 1) / (32 * (kSegThreads / 32));
         parts = (int)(most < kSegCtas * sms ? most : kSegCtas * sms);
         segment_fn(d)<<<parts, kSegThreads, osmem + 4, s>>>(points, N, d, K, centres, perm, start,
-                                                            d2_out, sums, partial);
+                                                            d2_out, sums, partial,
+                                                            reinterpret_cast<Control *>(ws));
     } else {
         parts = sms < L.grid ? sms : L.grid;
         ufn<<<parts, kUpdThreads, usmem, s>>>(points, N, d, K, centres, labels_out, d2_out, sums,

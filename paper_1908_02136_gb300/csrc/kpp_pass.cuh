@@ -647,6 +647,8 @@ template <int DT, int D, int L_, class RowAt, class Ahead, class Pre, class Sink
     static_assert(R * BB <= kPruneRing && (R & (R - 1)) == 0, "the ring holds them");
 
     const CentreRegs<DT, D, L_> &cr;
+    Control *ctl;         // debug build: index checks
+    int64_t base, nrows;  //   rows base + row_at() below nrows
     const char *src0;     // this lane's first vector of row 0 of the list's base
     const float *scales0; // its FP8 scale
     uint32_t ring, sring; // this lane's first vector; the FP8 scales of the rows in flight
@@ -660,10 +662,11 @@ template <int DT, int D, int L_, class RowAt, class Ahead, class Pre, class Sink
     int done = 0;     // groups consumed
     float part[G::L]; // this lane's share of each slot's row
 
-    __device__ __forceinline__ RowPipe(const PassIO &io, int64_t base,
+    __device__ __forceinline__ RowPipe(const PassIO &io, int64_t base_,
                                        const CentreRegs<DT, D, L_> &cr_, char *ring_, RowAt r,
                                        Ahead a, Pre p, Sink s)
-        : cr(cr_), row_at(r), ahead(a), pre(p), sink(s)
+        : cr(cr_), ctl(io.ctl), base(base_), nrows(io.bytes / G::RB), row_at(r), ahead(a), pre(p),
+          sink(s)
     {
         const int lane = threadIdx.x & 31;
         src0 = io.gpts + base * G::RB + (lane % G::L) * 16;
@@ -691,14 +694,15 @@ template <int DT, int D, int L_, class RowAt, class Ahead, class Pre, class Sink
         for (int q = 0; q < JB; ++q) {
             const char *src = src0 + (uint64_t)row[q] * G::RB;
             const int i = groups * 32 + (jb * JB + q) * (32 / G::L) + (int)(threadIdx.x & 31) / G::L;
-            if (!TAIL || i < n)
+            if ((!TAIL || i < n) && kpp_check(ctl, base + row[q] < nrows, 112))
 #pragma unroll
                 for (int v = 0; v < G::VPL; ++v)
                     cp_async16(dst + (q * G::VPL + v) * 512, src + v * G::L * 16);
         }
         if constexpr (DT == KPP_FP8_E4M3) {
             const int lane = threadIdx.x & 31;
-            if ((BR == 32 || lane < BR) && (!TAIL || groups * 32 + jb * BR + lane < n))
+            if ((BR == 32 || lane < BR) && (!TAIL || groups * 32 + jb * BR + lane < n) &&
+                kpp_check(ctl, base + row_at(groups * 32 + lane, jb * BR) < nrows, 113))
                 cp_async4(sring + (slot * BR + lane) * 4,
                           scales0 + row_at(groups * 32 + lane, jb * BR));
         }
@@ -823,6 +827,7 @@ template <int DT, class RowAt, class Ahead, class Pre, class Sink> struct Generi
     static constexpr int R = kPruneRing / BB; // batches in flight
     static_assert(R == 4, "four scale slots follow the ring");
 
+    Control *ctl; // debug build: index checks
     const char *pts;
     const float *scales;
     int64_t base;  // first row of the list's base
@@ -847,7 +852,8 @@ template <int DT, class RowAt, class Ahead, class Pre, class Sink> struct Generi
     __device__ __forceinline__ GenericPipe(const PassIO &io, int64_t base_, const float *cen_,
                                            int cen_lo_, char *ring_, RowAt r, Ahead a, Pre p,
                                            Sink s)
-        : pts(io.gpts), scales(io.scales), base(base_), bytes(io.bytes), cen(cen_), cen_lo(cen_lo_),
+        : ctl(io.ctl), pts(io.gpts), scales(io.scales), base(base_), bytes(io.bytes), cen(cen_),
+          cen_lo(cen_lo_),
           d(io.d), rb(io.d * EB), row_at(r), ahead(a), pre(p), sink(s)
     {
         // a row starts at a multiple of gcd(rb, 16) past a 32-byte boundary
@@ -884,6 +890,8 @@ template <int DT, class RowAt, class Ahead, class Pre, class Sink> struct Generi
                 // chunks from this one to the row's last (none past n); the
                 // last one of all points may be cut short
                 left[i] = TAIL && groups * 32 + (lane >> 2) + i * 8 >= n ? 0 : (ld + rb + 15) / 16 - j;
+                if (left[i] && !kpp_check(ctl, start >= 0 && start + rb <= bytes, 115))
+                    left[i] = 0;
                 const int64_t rem = bytes - at;
                 cut[i] = (int)(rem < (1 << 20) ? rem : (1 << 20));
             }
@@ -901,7 +909,8 @@ template <int DT, class RowAt, class Ahead, class Pre, class Sink> struct Generi
             }
         if (ib == 0 && (!TAIL || groups * 32 + lane < n))
             ahead(groups * 32 + lane);
-        if (DT == KPP_FP8_E4M3 && ib == 0 && (!TAIL || groups * 32 + lane < n))
+        if (DT == KPP_FP8_E4M3 && ib == 0 && (!TAIL || groups * 32 + lane < n) &&
+            kpp_check(ctl, (base + row_at(groups * 32 + lane, 0) + 1) * rb <= bytes, 116))
             cp_async4(sring + ((groups & 3) * 32 + lane) * 4,
                       scales + base + row_at(groups * 32 + lane, 0));
         cp_async_commit();
@@ -1207,7 +1216,8 @@ __device__ __forceinline__ void pass_rows_pruned(const PassIO &io, const PruneIO
         auto pipe = make_row_pipe<DT, D, L_>(
             io, seg_first, cr, pr.ring, [&](int i, int k) { return (uint32_t)at(i + k); },
             [&](int i) {
-                if (MODE == D2_INPLACE && !io.first)
+                if (MODE == D2_INPLACE && !io.first &&
+                    kpp_check(io.ctl, at(i) >= 0 && at(i) < rows, 117))
                     cp_async4((uint32_t)__cvta_generic_to_shared(old + i % kPruneList),
                               io.d2 + seg_first + at(i));
             },
