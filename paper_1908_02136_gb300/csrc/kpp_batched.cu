@@ -82,8 +82,7 @@ struct BatchPlan {
     std::vector<Wave> waves; // launched in this order
     // workspace layout
     size_t off_jobs, off_ctls, off_slots;
-    size_t min_bytes; // without the labels (such a workspace is accepted: every
-                      // pass then reads every row)
+    size_t min_bytes; // without the labels
     size_t off_labels, bytes;
     std::vector<size_t> slot_off; // per problem, relative to off_slots
     std::vector<size_t> lab_off;  // per problem, relative to off_labels (kNoLabels: none)
@@ -113,8 +112,9 @@ kpp_status check_problems(const kpp_problem *pr, int32_t n, int dt)
     return KPP_OK;
 }
 
+// labels: the workspace holds them, so that problems may skip rows.
 kpp_status make_batch_plan(const kpp_problem *pr, int32_t n, int dt, const kpp_options *opts,
-                           BatchPlan *bp)
+                           bool labels, BatchPlan *bp)
 {
     kpp_status st = check_problems(pr, n, dt);
     if (st != KPP_OK)
@@ -129,13 +129,24 @@ kpp_status make_batch_plan(const kpp_problem *pr, int32_t n, int dt, const kpp_o
     const int grid = sms; // one CTA per SM
     const int64_t min_rows = (opts && opts->min_rows_per_cta > 0) ? opts->min_rows_per_cta : 2048;
     const double eb = elem_bytes(dt);
+    // passes skip rows (kpp_pass.cuh) of at least 16 bytes
+    auto skips = [&](int i) {
+        return labels && pr[i].d * eb >= 16.0 && pr[i].K >= kBatchPruneMinK;
+    };
     // Cost model, in bytes at an SM's share of HBM: the share of the points a
     // pass reads once rows are skipped, D^2 and labels tested for every row,
     // and a fixed cost per pass (bounds, exchange and draw).  The 512-problem
     // batch takes 22.6 ms with the model of passes that read everything (1, 8
     // bytes; 64, 256 KB), 22.0 with 200 and 400 KB a pass, 21.4 with these.
+    // Problems that skip none are charged all they read.  Their share of the fixed
+    // cost is that of short chains (K < 8); batches of K = 4 and 200 mixed, ms as if
+    // they skipped / with 64, 256 KB / 300, 600 / these: FP32 29.0 / 28.4 / 28.5 / 28.2,
+    // BF16 18.4 / 16.7 / 16.5 / 16.6, FP8 20.4 / 20.0 / 19.5 / 19.1, 120 large ones 29.0 /
+    // 26.1 / 26.3 / 26.3; all K = 4 1.68 / 1.78 / 1.75 / 1.65.
     auto cost_of = [&](int i, int t) {
         const double rows = (double)pr[i].N / t;
+        if (!skips(i))
+            return (double)pr[i].K * (rows * (pr[i].d * eb + 8.0) + (t > 1 ? 1500.0e3 : 750.0e3));
         return (double)pr[i].K * (rows * (0.4 * pr[i].d * eb + 24.0) + (t > 1 ? 600.0e3 : 300.0e3));
     };
     std::vector<double> c1(n);
@@ -258,7 +269,7 @@ kpp_status make_batch_plan(const kpp_problem *pr, int32_t n, int dt, const kpp_o
     bp->lab_off.assign(n, kNoLabels);
     size_t loff = 0;
     for (int i = 0; i < n; ++i)
-        if (pr[i].d * eb >= 16.0 && pr[i].K >= kBatchPruneMinK) {
+        if (skips(i)) {
             bp->lab_off[i] = loff;
             loff += round_up(sizeof(uint16_t) * (size_t)pr[i].N, 64);
         }
@@ -277,7 +288,7 @@ size_t kpp_batch_workspace_size(const kpp_problem *problems, int32_t n, kpp_dtyp
                                 const kpp_options *opts)
 {
     BatchPlan bp;
-    if (make_batch_plan(problems, n, (int)dtype, opts, &bp) != KPP_OK)
+    if (make_batch_plan(problems, n, (int)dtype, opts, true, &bp) != KPP_OK)
         return 0;
     return bp.bytes;
 }
@@ -288,13 +299,17 @@ kpp_status kpp_seed_batched(const kpp_problem *problems, int32_t n, kpp_dtype dt
 {
     const int dt = (int)dtype;
     BatchPlan bp;
-    kpp_status st = make_batch_plan(problems, n, dt, opts, &bp);
+    kpp_status st = make_batch_plan(problems, n, dt, opts, true, &bp);
     if (st != KPP_OK)
         return st;
+    if (workspace_bytes < bp.bytes) { // no room for the labels: every row is read
+        st = make_batch_plan(problems, n, dt, opts, false, &bp);
+        if (st != KPP_OK)
+            return st;
+    }
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) % kAlign) != 0 ||
-        workspace_bytes < bp.min_bytes)
+        workspace_bytes < bp.bytes)
         return KPP_ERR_WORKSPACE;
-    const bool prune = workspace_bytes >= bp.bytes;
     char *ws = reinterpret_cast<char *>(workspace);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     // host image of the job table and the work lists
@@ -323,7 +338,7 @@ kpp_status kpp_seed_batched(const kpp_problem *problems, int32_t n, kpp_dtype dt
         p.nblocks = bp.nblocks[i];
         p.slots = reinterpret_cast<unsigned long long *>(ws + bp.off_slots + bp.slot_off[i]);
         p.exact_draws = (opts && opts->exact_draws) ? 1 : 0;
-        if (prune && bp.lab_off[i] != kNoLabels) {
+        if (bp.lab_off[i] != kNoLabels) {
             p.prune = 1;
             p.labels = reinterpret_cast<uint16_t *>(ws + bp.off_labels + bp.lab_off[i]);
         }
