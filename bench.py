@@ -119,10 +119,6 @@ KERNEL_SOURCES = {
 }
 
 
-# dynamic shared memory of the row rings and lists alone (16 warps)
-ROW_LIST_SMEM = 16 * (8192 + 512 + 2 * 512)
-
-
 def kernel_source_hash(kind: str = "persistent"):
     """SHA-256 over one kernel's CUDA sources (to tell whether a committed ncu
     traffic figure still describes the kernel being run)."""
@@ -487,7 +483,14 @@ def run_batch(args, rank, world, dev, pg, barrier):
     peaks = measured_peaks()
     peak = peaks["hbm_gbs"] if peaks else 6800.0
     # the slowest rank's own bytes over its own time would flatter; the
-    # roofline is per GPU: this rank's bytes over the job's step time
+    # roofline is per GPU: this rank's bytes over the job's step time.  The bytes
+    # read: points for the rows that are not skipped (K < 8 skip none, nor rows
+    # under 16 bytes, which the table has none of), D^2 and label of every row tested
+    all_bytes, alg_bytes = alg_bytes, 0.0
+    for x, pr, (idx, _, _) in zip(xs, table, outs):
+        r = rows_read(idx, x, None, pr.N, sample=1 << 11) if pr.K >= 8 else None
+        read, tests = r if r is not None else (pr.K, 0)
+        alg_bytes += read * pr.N * pr.d * 4 + 6.0 * pr.N * tests + 8.0 * pr.N * (pr.K - tests)
     achieved = alg_bytes / (ms / 1e3) / 1e9
     traffic = profiled_batch_traffic() if world == 1 else None
     if rank == 0:
@@ -508,6 +511,7 @@ def run_batch(args, rank, world, dev, pg, barrier):
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic,
                          "skips_rows": True,
+                         "equivalent": all_bytes / (ms / 1e3) / 1e9,
                          "kernel": "batched_kernel (all waves of one step)",
                          "algorithmic_bytes_per_launch": alg_bytes,
                          "algorithmic_bytes_all_ranks": alg_bytes_all},
@@ -660,8 +664,7 @@ def run_lloyd(args, rank, world, dev, pg, barrier):
                        "l2": "flushed between steps (512 MiB write)",
                        "phi": float(phi.item())},
             "clocks": clocks, "e2e": None,
-            # centres, assignment, update (count, order, walk; or one), means
-            "gpu_launches": (6 if N >= 200000 or N * d >= 10**7 else 4) * args.steps,
+            "gpu_launches": kpp.kpp_lloyd_launches(N, d, K) * args.steps,
             "roofline": {"bound": "tensor", "achieved": achieved, "peak": peak,
                          "unit": "TFLOP/s", "frac": achieved / peak, "traffic": None,
                          "kernel": "lloyd_assign_pair_kernel",
@@ -815,15 +818,66 @@ def read_peaks(kpp, dev):
     return out
 
 
+def rows_read(idx, pts, scales, rows_per_cta, launches=1, sample=1 << 16):
+    """(passes' worth of rows read, passes that test the rows) of a seeding whose
+    passes skip rows, estimated from evenly spaced points: their D^2 and nearest
+    seeds are followed through the passes with the kernels' bound
+    (4 D^2 <= (1 - 2^-8) |c - a|^2) and their rules for when a pass tests."""
+    import torch
+
+    K = idx.numel()
+    if int((idx < 0).any()):
+        return None
+    rows = torch.arange(0, pts.shape[0], max(1, pts.shape[0] // sample), device=pts.device)
+
+    def values(r):
+        v = pts[r]
+        if v.dtype == torch.int16:
+            return v.view(torch.bfloat16).float()
+        if v.dtype == torch.uint8:
+            return v.view(torch.float8_e4m3fn).float() * scales[r][:, None]
+        return v.float()
+
+    x, c = values(rows), values(idx)
+    d2 = (x - c[0]).square().sum(1)
+    lab = torch.zeros(len(rows), dtype=torch.int64, device=pts.device)
+    must = [torch.ones((), device=pts.device)]
+    for m in range(1, K):
+        s2 = (c[:min(m, 2048)] - c[m]).square().sum(1)
+        bound = torch.where(s2 < 1e-30, torch.zeros_like(s2), s2 * (0.25 * (1 - 2**-8)))
+        near = d2 <= bound[lab.clamp(max=len(bound) - 1)]
+        must.append(1.0 - (near & (lab < 2048)).float().mean())
+        v = (x - c[m]).square().sum(1)
+        lab = torch.where(v < d2, torch.full_like(lab, m), lab)
+        d2 = torch.minimum(d2, v)
+    must = torch.stack(must).tolist()
+    read, tests, few = 1.0, 0, False
+    decides = 8 * min(max(K // 128, 1), 128) + 1 if launches == 2 else 0
+    for m in range(1, K):
+        if not (few or (m % 8 == 1 and 4 * m <= rows_per_cta)):
+            read += 1.0
+            continue
+        tests += 1
+        read += must[m]
+        few = must[m] * rows_per_cta + m <= 0.8 * rows_per_cta
+        if m == decides and 1.0 - must[m] < 0.02:
+            read += K - 1 - m  # the kernel that reads every row goes on
+            break
+    return read, tests
+
+
 def roofline_for(plan, form_name, N, d, K, eb, has_scales, ms_per_step, wl_name, dtype, dev,
-                 peaks_live):
+                 peaks_live, skipped=None):
     """Roofline of the dominant kernel of one seeding (the persistent kernel,
     one launch per seeding, or the streamed pass kernel, K launches).
 
     Algorithmic bytes per pass = the points (N*d*b, plus 4N for FP8 scales),
     plus the 8N bytes of D^2 read and written where D^2 lives in global memory
     (streamed form; persistent form without room for D^2 in shared memory).
-    Plans whose passes skip rows read less (`skips_rows`).
+    Where passes skip rows (`skipped`, of rows_read) the points count for the
+    passes' worth of rows read, and D^2 in global memory and its 16-bit label for
+    the passes that test them; `equivalent` is then the rate at which passes over
+    all rows would have had to run.
     The bound is L2 when that working set fits the L2 (the persistent form
     keeps it there with an evict-last policy), HBM otherwise; `peak` is the
     measured copy bandwidth of MEASURED_PEAKS.json for HBM and the live
@@ -838,7 +892,11 @@ def roofline_for(plan, form_name, N, d, K, eb, has_scales, ms_per_step, wl_name,
     d2_global = form_name in ("streamed", "recompute") or not plan["d2_in_smem"]
     d2_bytes = 8 * N if d2_global else 0
     per_pass = point_bytes + d2_bytes
-    alg_bytes = passes_per_launch * per_pass
+    alg_bytes = all_bytes = passes_per_launch * per_pass
+    if skipped is not None:
+        read, tests = skipped
+        alg_bytes = int(read * point_bytes + (0 if plan["d2_in_smem"] else
+                                              6 * N * tests + 8 * N * (K - tests)))
     achieved = alg_bytes / (per_launch_ms / 1e3) / 1e9
     working_set = point_bytes + (4 * N if d2_global else 0)
     l2 = l2_bytes(dev)
@@ -865,12 +923,12 @@ def roofline_for(plan, form_name, N, d, K, eb, has_scales, ms_per_step, wl_name,
         r["l2_read_gbs"] = peaks_live["l2_read_gbs"]
     if traffic is not None:
         r["traffic_over_algorithmic"] = traffic / alg_bytes
-    # persistent plans without a point cache but with the row lists' shared
-    # memory skip the rows a new seed cannot bring nearer (exactly: D^2 and the
-    # draws keep every bit), so these bytes are what passes over all points
-    # would read: `achieved` is an equivalent rate and may exceed the peak
-    r["skips_rows"] = (form_name == "persistent" and plan["cached_rows_per_cta"] == 0 and
-                       plan["smem_bytes"] >= ROW_LIST_SMEM)
+    # rows a new seed cannot bring nearer are left out (exactly: D^2 and the draws
+    # keep every bit)
+    r["skips_rows"] = skipped is not None
+    if skipped is not None:
+        r["rows_read"] = skipped[0] / K
+        r["equivalent"] = all_bytes / (per_launch_ms / 1e3) / 1e9
     return r
 
 
@@ -1025,8 +1083,18 @@ def run_seeding(args, rank, world, local, dev, pg, barrier):
     ms_per_step = main_r["ms"]
     nkd = float(N) * K * d
     value = nkd * world / (ms_per_step / 1e3)
-    roofline = roofline_for(main_r["plan"], main_r["form"], N, d, K, ebytes[dtype],
-                            scales is not None, ms_per_step, wl.name, dtype, dev, peaks_live)
+
+    def skipped(r):
+        if not kpp.kpp_skips_rows(N, d, K, codes[r["dtype"]], opts):
+            return None
+        return rows_read(r["idx"], r["pts"], r["scales"], r["plan"]["rows_per_cta"],
+                         r["plan"]["launches"])
+
+    main_r["dtype"] = dtype
+    with torch.cuda.device(dev):
+        roofline = roofline_for(main_r["plan"], main_r["form"], N, d, K, ebytes[dtype],
+                                scales is not None, ms_per_step, wl.name, dtype, dev, peaks_live,
+                                skipped(main_r))
     precision = None
     if dtype != "f32" and not args.no_phi:
         precision = phi_gate(dtype, main_r)
@@ -1043,9 +1111,10 @@ def run_seeding(args, rank, world, local, dev, pg, barrier):
             fpts, fsc, fq_ms = store(fd)
             fr = time_form(fd, fpts, fsc, max(1, min(args.steps, args.form_steps)),
                            max(1, min(args.warmup, 2)))
-            fr["pts"], fr["scales"] = fpts, fsc
-            froof = roofline_for(fr["plan"], fr["form"], N, d, K, ebytes[fd], fsc is not None,
-                                 fr["ms"], wl.name, fd, dev, peaks_live)
+            fr["pts"], fr["scales"], fr["dtype"] = fpts, fsc, fd
+            with torch.cuda.device(dev):
+                froof = roofline_for(fr["plan"], fr["form"], N, d, K, ebytes[fd], fsc is not None,
+                                     fr["ms"], wl.name, fd, dev, peaks_live, skipped(fr))
             entry = {"ms_per_seeding": fr["ms"], "value": nkd * world / (fr["ms"] / 1e3),
                      "speedup_vs_f32": ms_per_step / fr["ms"], "steps": fr["steps"],
                      "quantize_ms": fq_ms, "form": fr["form"], "plan": fr["plan"],
@@ -1055,7 +1124,8 @@ def run_seeding(args, rank, world, local, dev, pg, barrier):
                                   ("bound", "achieved", "peak", "frac", "traffic",
                                    "traffic_over_algorithmic", "frac_of_hbm_read",
                                    "frac_of_nominal_hbm", "us_per_pass",
-                                   "algorithmic_bytes_per_pass", "skips_rows")
+                                   "algorithmic_bytes_per_pass", "skips_rows", "rows_read",
+                                   "equivalent")
                                   if k in froof}}
             if not args.no_phi:
                 entry["phi"] = phi_gate(fd, fr)

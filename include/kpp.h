@@ -183,6 +183,14 @@ KPP_API kpp_status kpp_describe(int64_t N, int32_t d, int32_t K, kpp_dtype dtype
                                 const kpp_options *opts, kpp_plan *plan);
 
 /*
+ * 1 if the passes of kpp_seed leave out rows they cannot change under the plan
+ * for these arguments (given kpp_workspace_size bytes of workspace), else 0
+ * (also for invalid arguments).  Host-side only.
+ */
+KPP_API int32_t kpp_skips_rows(int64_t N, int32_t d, int32_t K, kpp_dtype dtype,
+                               const kpp_options *opts);
+
+/*
  * k-means++ seeding of one problem (Algorithm 1 / Algorithm 2).
  *   points        [N x d] stored values of `dtype`, 16-byte aligned
  *   row_scales    [N] FP32 per-row scales (KPP_FP8_E4M3 only, else NULL)
@@ -382,6 +390,9 @@ KPP_API void kpp_tune_clear(void);
  * one-SM kernel.  Both give the same labels.
  */
 KPP_API size_t kpp_lloyd_workspace_size(int64_t N, int32_t d, int32_t K);
+/* Kernel launches of one kpp_lloyd_step in a workspace of that size (0 if the
+ * arguments are invalid). */
+KPP_API int32_t kpp_lloyd_launches(int64_t N, int32_t d, int32_t K);
 KPP_API kpp_status kpp_lloyd_prepare(const float *points, int64_t N, int32_t d, int32_t K,
                                      void *workspace, size_t workspace_bytes,
                                      kpp_stream_t stream);

@@ -121,6 +121,8 @@ def load_library(build_if_stale: bool = True):
         lib.kpp_workspace_size.restype = ctypes.c_size_t
         lib.kpp_describe.argtypes = [I64, I32, I32, ctypes.c_int, P, P]
         lib.kpp_describe.restype = ctypes.c_int
+        lib.kpp_skips_rows.argtypes = [I64, I32, I32, ctypes.c_int, P]
+        lib.kpp_skips_rows.restype = I32
         lib.kpp_seed.argtypes = [P, P, I64, I32, I32, ctypes.c_int, U64, U64, P, I32, P, P, P,
                                  P, ctypes.c_size_t, P, P]
         lib.kpp_seed.restype = ctypes.c_int
@@ -161,6 +163,8 @@ def load_library(build_if_stale: bool = True):
         lib.kpp_tune_clear.restype = None
         lib.kpp_lloyd_workspace_size.argtypes = [I64, I32, I32]
         lib.kpp_lloyd_workspace_size.restype = ctypes.c_size_t
+        lib.kpp_lloyd_launches.argtypes = [I64, I32, I32]
+        lib.kpp_lloyd_launches.restype = I32
         lib.kpp_lloyd_prepare.argtypes = [P, I64, I32, I32, P, ctypes.c_size_t, P]
         lib.kpp_lloyd_prepare.restype = ctypes.c_int
         lib.kpp_lloyd_step.argtypes = [P, I64, I32, P, I32, P, P, P, P, P, P, ctypes.c_size_t, P]
@@ -210,6 +214,11 @@ def kpp_describe(N, d, K, dtype, opts=None, plan=None):
     plan = plan if plan is not None else Plan()
     st = load_library().kpp_describe(N, d, K, dtype, _opts_ptr(opts), ctypes.byref(plan))
     return st, plan
+
+
+def kpp_skips_rows(N, d, K, dtype, opts=None) -> bool:
+    """Whether passes of kpp_seed leave out rows under the plan for these arguments."""
+    return bool(load_library().kpp_skips_rows(N, d, K, dtype, _opts_ptr(opts)))
 
 
 def kpp_seed(points, row_scales, N, d, K, dtype, seed, stream_id, forced_prefix, n_forced,
@@ -386,6 +395,10 @@ def kpp_tune_clear() -> None:
 
 def kpp_lloyd_workspace_size(N, d, K) -> int:
     return load_library().kpp_lloyd_workspace_size(N, d, K)
+
+
+def kpp_lloyd_launches(N, d, K) -> int:
+    return load_library().kpp_lloyd_launches(N, d, K)
 
 
 def kpp_lloyd_prepare(points, N, d, K, workspace, workspace_bytes, stream) -> int:

@@ -692,6 +692,12 @@ kpp_status kpp_describe(int64_t N, int32_t d, int32_t K, kpp_dtype dtype,
     return KPP_OK;
 }
 
+int32_t kpp_skips_rows(int64_t N, int32_t d, int32_t K, kpp_dtype dtype, const kpp_options *opts)
+{
+    PlanFacts f;
+    return plan_facts(N, d, K, dtype, opts, &f) == KPP_OK && f.skips ? 1 : 0;
+}
+
 kpp_status kpp_seed(const void *points, const float *row_scales, int64_t N, int32_t d,
                     int32_t K, kpp_dtype dtype, uint64_t seed, uint64_t stream_id,
                     const int64_t *forced_prefix, int32_t n_forced, int64_t *indices_out,

@@ -1564,6 +1564,14 @@ size_t kpp_lloyd_workspace_size(int64_t N, int32_t d, int32_t K)
     return layout(N, d, K).bytes;
 }
 
+int32_t kpp_lloyd_launches(int64_t N, int32_t d, int32_t K)
+{
+    if (!shape_ok(N, d, K))
+        return 0;
+    // the centres, the assignment, the update (count, order, walk; or one), the means
+    return 3 + (update_ordered(N, d, K) ? 3 : 1);
+}
+
 kpp_status kpp_lloyd_prepare(const float *points, int64_t N, int32_t d, int32_t K, void *workspace,
                              size_t workspace_bytes, kpp_stream_t stream)
 {

@@ -93,3 +93,20 @@ def test_plans_that_read_every_row_can_be_asked_for(N, d, dtype):
         assert plan.d2_in_smem == (plan.rows_per_cta * 4.25 < 220 * 1024)
         out = kpp.seed(x, K, 3, row_scales=scales, opts=opts)
         assert torch.equal(ref[0], out[0]) and torch.equal(ref[1], out[1])
+
+
+def test_what_a_plan_skips_and_launches():
+    """kpp_skips_rows and kpp_lloyd_launches on both sides of their rules."""
+    for N, d, K, opts, skips in [(300_000, 64, 24, None, True), (300_000, 64, 7, None, False),
+                                 (300_000, 64, 24, {"form": 2, "smem_cache": -2}, False),
+                                 (300_000, 2, 24, None, False), (9_000, 2, 24, None, False),
+                                 (6_000_000, 8, 100, {"form": 2, "smem_cache": 1 << 30}, False),
+                                 (300_000, 50, 24, None, True), (5_000_000, 100, 6, None, False),
+                                 (300_000, 64, 24, {"form": kpp.FORM_STREAMED}, False)]:
+        assert kpp.kpp_skips_rows(N, d, K, kpp.F32, opts) == skips, (N, d, K, opts)
+    assert not kpp.kpp_skips_rows(10, 8, 11, kpp.F32)
+    # the update over ordered points: many points, many values, or many centre tiles
+    for N, d, K, n in [(199_999, 8, 20, 4), (200_000, 8, 20, 6), (104_166, 96, 50, 4),
+                       (104_167, 96, 50, 6), (7_812, 128, 2000, 4), (7_813, 128, 2000, 6)]:
+        assert kpp.kpp_lloyd_launches(N, d, K) == n, (N, d, K)
+    assert kpp.kpp_lloyd_launches(10, 200, 5) == 0
