@@ -1277,8 +1277,8 @@ bool update_ordered(int64_t N, int d, int K)
 using SegmentFn = void (*)(const float *, int64_t, int, int, const float *, const int32_t *,
                            const int32_t *, float *, double *, double *, Control *);
 
-// Lanes per row by d, so that few lanes idle; 64 rows' worth of loads or 8 KB
-// a warp in flight.
+// Lanes per row by d, so that few lanes idle; in flight a warp has 128 rows
+// (d <= 4) down to 8 (d > 64): at most 2 KB to d = 32, 4 KB above.
 SegmentFn segment_fn(int d)
 {
     if (d <= 4)

@@ -571,9 +571,15 @@ __device__ __forceinline__ Pair pass_rows(const PassIO &io, const CentreRegs<DT,
 // last).  Whole seedings before and after: 10^7 x 64, K = 1024 FP32 381 -> 152
 // ms, BF16 225 -> 92 ms; 2 10^7 x 128, K = 2048 FP8 1337 -> 506 ms; 10^6 x 32,
 // K = 256 (in L2) 3.90 -> 3.00 ms; the 512-problem batch 40.6 -> 22.7 ms.
-// Passes that read every row cost what they do in the plain kernel (10^7 x 64,
-// K = 8 without clusters: 3.12 / 3.13 ms; 10^6 x 32: 130 / 140 us), FP8 ones less
-// (2 10^7 x 128: 0.49 / 0.65 ms a pass).
+// What data without clusters pays, where no row is ever skipped (normal
+// coordinates, ms with every row read / so): far beyond L2 nothing (10^7 x 64,
+// K = 64 24.6 / 24.5), narrow and FP8 rows gain from the row pipe (10^7 x 16 8.8 / 6.9,
+// 10^6 x 128 FP8, K = 100 3.39 / 3.06), sets in L2 gain a little (10^6 x 32, K = 256
+// 3.91 / 3.78; 2 10^5 x 32 1.84 / 1.85).  Where the lists push D^2 out of shared
+// memory (1.6 to 8 10^6 points) rows of 128 bytes and more lose 1 to 4 % from 20 GB
+// of rows in all passes on, where the plain kernel stands by (kpp_persistent.cuh;
+// 2 10^6 x 64, K = 128 9.17 / 9.32, 4 10^6 x 32, K = 64 4.69 / 4.87), and up to 10 % in
+// shorter seedings, which in clusters gain as much.
 // ---------------------------------------------------------------------------
 constexpr int kPruneCentres = 2048; // centres with a bound; rows of later ones are always read
 constexpr uint16_t kNoLabel = 0xffff;
