@@ -321,8 +321,8 @@ KPP_API kpp_status kpp_seed_batched(const kpp_problem *problems, int32_t n, kpp_
  * CUDA events on `stream`; candidates are tried defaults first, and a later one
  * replaces the best so far only if it is more than 1 % faster.  The best plan
  * whose passes skip rows and the best that reads every row are then compared
- * over one whole seeding each, since what is skipped depends on the data and
- * grows with the seeds.
+ * over one whole seeding each (4096 passes at most), since what is skipped
+ * depends on the data and grows with the seeds.
  *   points, row_scales, N, d, K, dtype   as for kpp_seed
  *   indices_out [K], d2_out [N]          device scratch for the trial runs
  *                                        (their contents are undefined after)

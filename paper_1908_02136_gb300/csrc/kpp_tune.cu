@@ -328,14 +328,17 @@ kpp_status kpp_tune(const void *points, const float *row_scales, int64_t N, int3
     // K = 1024 in clusters: 0.39 ms a pass falling to 0.03) or not, as the data
     // has it (2 10^6 x 64, K = 256 in clusters: 32 passes still favour the plan
     // that reads every row, which takes 18.1 ms in all for 8.9).  So each of the
-    // two winners takes a whole seeding.
+    // two winners takes a whole seeding, of kMostPasses passes at most: from the
+    // 2 049th seed on there are no more bounds, and no more to learn.
     int win = kind[1].ms > 0.f && (kind[0].ms < 0.f || kind[1].order < kind[0].order) ? 1 : 0;
     if (result == KPP_OK && kind[0].ms > 0.f && kind[1].ms > 0.f) {
+        constexpr int32_t kMostPasses = 4096;
+        const int32_t Kf = std::min(K, std::max(Kt, kMostPasses));
         float ms[2] = {kind[0].ms, kind[1].ms};
-        for (int k = 0; K > Kt && k < 2; ++k) {
+        for (int k = 0; Kf > Kt && k < 2; ++k) {
             float t;
             const kpp_status st =
-                time_passes(kind[k].o, K, kind[k].o.form == KPP_FORM_STREAMED, 1, &t);
+                time_passes(kind[k].o, Kf, kind[k].o.form == KPP_FORM_STREAMED, 1, &t);
             if (st == KPP_ERR_CUDA)
                 result = st;
             // (fewer distinct points than K: the first passes decide)

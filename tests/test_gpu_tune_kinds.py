@@ -115,3 +115,11 @@ def test_a_recorded_streamed_choice_stands_for_any_d(tmp_path):
                        env=dict(os.environ, KPP_TUNE_CACHE=str(cache)), timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
     assert json.loads(r.stdout.strip().splitlines()[-1]) == [kpp.OK, kpp.FORM_STREAMED]
+
+
+def test_more_seeds_than_the_tuner_runs():
+    """K = N: the whole seedings that decide stop at 4096 passes."""
+    N, d = 20_011, 64
+    x = torch.from_numpy(datagen.gmm(N, d, 64, seed=3)).to(DEV)
+    best, ms = kpp.tune(x, N, passes=8)
+    assert best["form"] in (kpp.FORM_STREAMED, kpp.FORM_PERSISTENT) and ms > 0
